@@ -42,11 +42,21 @@ struct Px;
 
 template <>
 struct Px<DFB_F32> {
+  using Raw = float4;
+  static __device__ __forceinline__ Raw raw(const unsigned char* base, int p) {
+    return reinterpret_cast<const float4*>(base)[p];
+  }
+  static __device__ __forceinline__ float4 decode(Raw v, float) { return v; }
+  // zero exactly when every stored bit is zero
+  static __device__ __forceinline__ uint32_t bits(Raw v) {
+    return __float_as_uint(v.x) | __float_as_uint(v.y) | __float_as_uint(v.z) |
+           __float_as_uint(v.w);
+  }
   static __device__ __forceinline__ float4 global(const void* base, int p, float) {
     return __ldg(reinterpret_cast<const float4*>(base) + p);
   }
   static __device__ __forceinline__ float4 shared(const unsigned char* base, int p, float) {
-    return reinterpret_cast<const float4*>(base)[p];
+    return raw(base, p);
   }
 };
 
@@ -59,11 +69,17 @@ __device__ __forceinline__ float4 decode_f16(uint2 v) {
 
 template <>
 struct Px<DFB_F16> {
+  using Raw = uint2;
+  static __device__ __forceinline__ Raw raw(const unsigned char* base, int p) {
+    return reinterpret_cast<const uint2*>(base)[p];
+  }
+  static __device__ __forceinline__ float4 decode(Raw v, float) { return decode_f16(v); }
+  static __device__ __forceinline__ uint32_t bits(Raw v) { return v.x | v.y; }
   static __device__ __forceinline__ float4 global(const void* base, int p, float) {
     return decode_f16(__ldg(reinterpret_cast<const uint2*>(base) + p));
   }
   static __device__ __forceinline__ float4 shared(const unsigned char* base, int p, float) {
-    return decode_f16(reinterpret_cast<const uint2*>(base)[p]);
+    return decode_f16(raw(base, p));
   }
 };
 
@@ -74,11 +90,17 @@ __device__ __forceinline__ float4 decode_bf16(uint2 v) {
 
 template <>
 struct Px<DFB_BF16> {
+  using Raw = uint2;
+  static __device__ __forceinline__ Raw raw(const unsigned char* base, int p) {
+    return reinterpret_cast<const uint2*>(base)[p];
+  }
+  static __device__ __forceinline__ float4 decode(Raw v, float) { return decode_bf16(v); }
+  static __device__ __forceinline__ uint32_t bits(Raw v) { return v.x | v.y; }
   static __device__ __forceinline__ float4 global(const void* base, int p, float) {
     return decode_bf16(__ldg(reinterpret_cast<const uint2*>(base) + p));
   }
   static __device__ __forceinline__ float4 shared(const unsigned char* base, int p, float) {
-    return decode_bf16(reinterpret_cast<const uint2*>(base)[p]);
+    return decode_bf16(raw(base, p));
   }
 };
 
@@ -90,11 +112,19 @@ __device__ __forceinline__ float4 decode_fp8(uint32_t v, float scale) {
 
 template <>
 struct Px<DFB_FP8E4M3> {
+  using Raw = uint32_t;
+  static __device__ __forceinline__ Raw raw(const unsigned char* base, int p) {
+    return reinterpret_cast<const unsigned int*>(base)[p];
+  }
+  static __device__ __forceinline__ float4 decode(Raw v, float scale) {
+    return decode_fp8(v, scale);
+  }
+  static __device__ __forceinline__ uint32_t bits(Raw v) { return v; }
   static __device__ __forceinline__ float4 global(const void* base, int p, float scale) {
     return decode_fp8(__ldg(reinterpret_cast<const unsigned int*>(base) + p), scale);
   }
   static __device__ __forceinline__ float4 shared(const unsigned char* base, int p, float scale) {
-    return decode_fp8(reinterpret_cast<const unsigned int*>(base)[p], scale);
+    return decode_fp8(raw(base, p), scale);
   }
 };
 
