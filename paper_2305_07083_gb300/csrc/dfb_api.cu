@@ -612,11 +612,12 @@ bool valid_tuning(int ring_kb, int ctas_per_sm, int groups) {
   return false;
 }
 
-// Launch shape for a launch of `nRec` fragment tiles over `nTiles` tiles.
-dfb::TuneParams tune_of(const dfb_ctx* h, size_t nRec, size_t nTiles) {
+// Launch shape for a launch of one frame or several, `nRec` fragment tiles
+// over `nTiles` tiles.
+dfb::TuneParams tune_of(const dfb_ctx* h, size_t nRec, size_t nTiles, bool oneFrame) {
   return h->tune.ringKB ? h->tune
                         : dfb::default_tune(h->cfg.dtype,
-                                            (double)nRec / (double)(nTiles ? nTiles : 1));
+                                            (double)nRec / (double)(nTiles ? nTiles : 1), oneFrame);
 }
 
 dfb::LaunchCtl ctl_of(const dfb_ctx* h, int* redo) {
@@ -1180,7 +1181,7 @@ int end_one(dfb_ctx* h, cudaStream_t s) {
   if (e == cudaSuccess)
     e = dfb::launch_composite(dFa, dItemBase, 1, items, h->nTiles,
                               (h->cfg.flags & DFB_FLAG_ACCUMULATE) != 0, h->cfg.dtype,
-                              tune_of(h, n, (size_t)h->nTiles),
+                              tune_of(h, n, (size_t)h->nTiles, true),
                               ctl_of(h, b.redo), lng, &hdr->fa, hdr->itemBase,
                               ev ? ev[3] : nullptr, s);
   if (e == cudaSuccess) e = cudaEventRecord(b.released, s);
@@ -1277,7 +1278,7 @@ int end_batch(dfb_ctx* const* hs, int n, cudaStream_t s) {
   if (e == cudaSuccess && ev) e = cudaEventRecord(ev[2], s);
   if (e == cudaSuccess)
     e = dfb::launch_composite(b.dFrames, b.dItemBase, n, items, tileBase, anyAcc, dtype,
-                              tune_of(hs[0], nRec, nTiles), ctl_of(hs[0], b.redo), lng, b.hFrames,
+                              tune_of(hs[0], nRec, nTiles, false), ctl_of(hs[0], b.redo), lng, b.hFrames,
                               b.hItemBase,
                               ev ? ev[3] : nullptr, s);
   if (e == cudaSuccess) e = cudaEventRecord(b.released, s);
@@ -1615,12 +1616,15 @@ void graph_release_capture(dfb_graph_t* g) {
   g->graph = nullptr;
 }
 
+dfb::TuneParams default_graph_tune(const dfb_graph_t* g) {
+  return dfb::default_tune(g->dtype, (double)g->nRec / (double)(g->nTiles ? g->nTiles : 1),
+                           g->hs.size() == 1);
+}
+
 // (Re)capture the device work of the graph with its current tuning.
 int graph_capture(dfb_graph_t* g) {
   graph_release_capture(g);
-  const dfb::TuneParams tune =
-      g->tune.ringKB ? g->tune
-                     : dfb::default_tune(g->dtype, (double)g->nRec / (double)(g->nTiles ? g->nTiles : 1));
+  const dfb::TuneParams tune = g->tune.ringKB ? g->tune : default_graph_tune(g);
   // per-device launch set-up happens outside the capture (no work is enqueued)
   const dfb::LaunchCtl ctl{2000000000ull, -1, g->err, g->redo};
   cudaError_t e = dfb::launch_composite(g->dFrames, g->dItemBase, 1, 0, 0, false, g->dtype, tune,
@@ -1834,8 +1838,7 @@ int dfb_graph_autotune(dfb_graph g, void* stream, int reps, int* ring_kb, int* c
     cudaError_t e = cudaEventCreate(&a);
     if (e == cudaSuccess) e = cudaEventCreate(&b);
     float best = 1e30f;
-    dfb::TuneParams bestT =
-        dfb::default_tune(g->dtype, (double)g->nRec / (double)(g->nTiles ? g->nTiles : 1));
+    dfb::TuneParams bestT = default_graph_tune(g);
     for (const auto& c : cand) {
       if (e != cudaSuccess) break;
       if (dfb_graph_set_tuning(g, c[0], c[1], c[2]) != DFB_OK) continue;  // does not fit

@@ -1216,16 +1216,20 @@ cudaError_t launch_dt(const FrameArgs* frames, const int* itemBase, int nFrames,
 
 }  // namespace
 
-// Measured (composite launch, 16-frame accumulation): FP32 takes 2 CTAs per
-// SM with one consumer group each and the largest ring they share.  The
-// narrower formats fit their fills into the rings of 3 CTAs per SM, which is
-// faster unless the frames are fragment-heavy: FP16 at 5.5 fragments per
-// tile 0.1058 ms with 2 CTAs against 0.1095 ms with 3; at 4.4 fragments per
-// tile 0.1028 against 0.0945 ms; at one fragment per tile 3 CTAs are faster
-// too.  One CTA per SM is slower everywhere: its single producer warp sets
-// the pace.
-TuneParams default_tune(int dtype, double fragmentsPerTile) {
-  if (dtype == DFB_F32 || fragmentsPerTile >= 5.0) return TuneParams{110, 2, 1};
+// Measured (composite launch): FP32 takes 2 CTAs per SM with one consumer
+// group each and the largest ring they share; its largest fill does not fit
+// the rings of 3.  The narrower formats' does, and 3 CTAs per SM are faster:
+// FP8 4096x1024, 3.4 fragments per tile, accumulating, 82 against 88 us; 16
+// mixed FP16 frames of 2 to 25 per tile in one launch 634 against 708 us.  The
+// exception is a single fragment-heavy frame, where the 2-CTA shape loads the
+// state one item ahead: FP16 2048x2048, 5.5 per tile, accumulating, 102.0
+// against 107.3 us (4.4 per tile: 102.8 against 94.5).  There a ring of 70 KB
+// beats the largest (103.6 us): more reads in flight than the DRAM queues
+// need only spread the accesses to a tile in time.  One CTA per SM is slower
+// everywhere: its single producer warp sets the pace.
+TuneParams default_tune(int dtype, double fragmentsPerTile, bool oneFrame) {
+  if (dtype == DFB_F32) return TuneParams{110, 2, 1};
+  if (oneFrame && fragmentsPerTile >= 5.0) return TuneParams{70, 2, 1};
   return TuneParams{72, 3, 1};
 }
 

@@ -165,10 +165,9 @@ cudaError_t launch_composite(const FrameArgs* frames, const int* itemBase, int n
                              const FrameArgs* hostFrames, const int* hostItemBase,
                              cudaEvent_t afterMain, cudaStream_t s);
 
-// Default launch shape for a dtype.
-// Default launch shape for a launch whose frames have `fragmentsPerTile`
-// fragment tiles per image tile on average.
-TuneParams default_tune(int dtype, double fragmentsPerTile);
+// Default launch shape for a launch of one frame or several, with
+// `fragmentsPerTile` fragment tiles per image tile on average.
+TuneParams default_tune(int dtype, double fragmentsPerTile, bool oneFrame);
 
 // Mean fragments per tile from which the composite's consumers load a
 // frame's accumulation state themselves instead of receiving it through the

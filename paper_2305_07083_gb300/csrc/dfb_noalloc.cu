@@ -305,7 +305,7 @@ int composite_noalloc(int width, int height, int tile_size, int mode, int dtype,
   if (e != cudaSuccess) return DFB_ERR_CUDA;
   const dfb::LaunchCtl ctl{g_waitNs.load(), g_stallItem.exchange(-1), &dHdr->err, redo};
   e = dfb::launch_composite(&dHdr->fa, dHdr->itemBase, 1, hdr.itemBase[1], nTiles, false, dtype,
-                           dfb::default_tune(dtype, (double)n / (double)nTiles), ctl, lng,
+                           dfb::default_tune(dtype, (double)n / (double)nTiles, true), ctl, lng,
                            &hdr.fa, hdr.itemBase, nullptr, s);
   if (e != cudaSuccess) return DFB_ERR_CUDA;
   // The launch's error word: a wait that ran out (the frame is then
