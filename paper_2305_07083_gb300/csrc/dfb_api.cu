@@ -118,6 +118,7 @@ struct dfb_ctx {
   int tilesX = 0, tilesY = 0, nTiles = 0, logT = 0, chunks = 0, tilePixels = 0;
   size_t rgbaBytes = 0, depthBytes = 0;
   int device = 0;
+  int l2Bytes = 0;
   bool allocated = false;
 
   // frame state
@@ -363,6 +364,8 @@ int allocate(dfb_ctx* h) {
   if (h->allocated) return dev == h->device ? DFB_OK : DFB_ERR_STATE;
   if (h->curve && dev != h->curveDevice) return DFB_ERR_STATE;
   h->device = dev;
+  if (cudaDeviceGetAttribute(&h->l2Bytes, cudaDevAttrL2CacheSize, dev) != cudaSuccess)
+    return DFB_ERR_CUDA;
   int st = ensure_table(dev);
   if (st != DFB_OK) return st;
   const size_t px = (size_t)h->cfg.width * h->cfg.height;
@@ -560,6 +563,19 @@ int check_trees(const dfb_ctx* h) {
   return DFB_OK;
 }
 
+// Tiles of the open frame whose state stays in L2 (FrameArgs::keepTiles), for
+// `statePx` bytes of state per pixel: all of them, and no streaming, where a
+// frame's bytes are no more than half of L2 or there is no state.
+int keep_tiles(const dfb_ctx* h, int statePx) {
+  if (!(h->cfg.flags & DFB_FLAG_ACCUMULATE)) return dfb::kKeepAll;
+  const double px = (double)h->nTiles * h->tilePixels;
+  const double bytes = (double)h->recs.size() * (double)(h->rgbaBytes + h->depthBytes) +
+                       px * (statePx + ((h->cfg.flags & DFB_FLAG_WRITE_COLOR) ? 16 : 0) +
+                             ((h->cfg.flags & DFB_FLAG_PACK_RGBA8) ? 4 : 0));
+  if (bytes <= 0.5 * h->l2Bytes) return dfb::kKeepAll;
+  return (int)(dfb::kKeepFraction * h->l2Bytes / ((double)statePx * h->tilePixels));
+}
+
 void fill_frame_args(const dfb_ctx* h, FrameArgs& a, int tileBase, const FragRec* srecs,
                      const dfb::TileBlock* blocks) {
   dfb::frame_geometry(a, h->cfg.width, h->cfg.height, h->cfg.tile_size);
@@ -591,6 +607,7 @@ void fill_frame_args(const dfb_ctx* h, FrameArgs& a, int tileBase, const FragRec
   // (FP32 at 5.5 fragments per tile: 0.1279 ms against 0.1302 ms).
   a.stateInRing =
       (double)h->recs.size() < dfb::kStateLoadFragmentsPerTile * (double)h->nTiles ? 1 : 0;
+  a.keepTiles = keep_tiles(h, a.kahan ? 48 : 32);
   a.srecs = srecs;
   a.blocks = blocks;
   a.color = h->color;

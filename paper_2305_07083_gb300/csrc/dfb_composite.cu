@@ -135,6 +135,9 @@ struct FrameTable {
   FrameArgs f[kParamFrames];
 };
 static_assert(sizeof(FrameTable) <= 16384, "kernel parameter size");
+// Whether a launch's frames choose what stays in L2 (FrameArgs::keepTiles).
+template <int FR>
+constexpr bool kKeeps = FR == kOneFrame;
 template <int FR>
 struct FrameParams {
   using type = int;  // unused
@@ -265,6 +268,7 @@ __device__ void producer(const FrameArgs* __restrict__ frames, const int* __rest
     Sizes sz;
   };
   const Sizes one = FR == kOneFrame ? sizes(frames) : Sizes{};
+  const uint64_t evictFirst = l2_evict_first();
   int scanF = 0;
   auto plan = [&](int r) -> Plan {
     Plan p{};
@@ -417,7 +421,12 @@ __device__ void producer(const FrameArgs* __restrict__ frames, const int* __rest
           armed |= 1u << s;
           armedPar = (armedPar & ~(1u << s)) | (par << s);
           __syncwarp();
-          if (lane < nf) {
+          if (kKeeps<FR> && A->keepTiles != kKeepAll) {
+            if (lane < nf) {
+              if (dBytes) bulk_g2s_hint(dDst, dSrc, dBytes, &fullB[s], evictFirst);
+              if (cBytes) bulk_g2s_hint(cDst, cSrc, cBytes, &fullB[s], evictFirst);
+            }
+          } else if (lane < nf) {
             if (dBytes) bulk_g2s(dDst, dSrc, dBytes, &fullB[s]);
             if (cBytes) bulk_g2s(cDst, cSrc, cBytes, &fullB[s]);
           }
@@ -427,8 +436,12 @@ __device__ void producer(const FrameArgs* __restrict__ frames, const int* __rest
                 FR == kOneFrame ? item >> A->logChunks : __shfl_sync(0xffffffffu, cur.tile, u);
             if (lane < nState) {
               const float4* src = lane == 0 ? A->accum : (lane == 1 ? A->m2 : A->comp);
-              bulk_g2s(ring + start + fragBytes + lane * (uint32_t)P * 16u,
-                       src + (size_t)tile * A->T * A->T + p0, (uint32_t)P * 16u, &fullB[s]);
+              void* dst = ring + start + fragBytes + lane * (uint32_t)P * 16u;
+              src += (size_t)tile * A->T * A->T + p0;
+              if (kKeeps<FR> && tile >= A->keepTiles)
+                bulk_g2s_hint(dst, src, (uint32_t)P * 16u, &fullB[s], evictFirst);
+              else
+                bulk_g2s(dst, src, (uint32_t)P * 16u, &fullB[s]);
             }
           }
         }
@@ -697,11 +710,18 @@ __device__ __forceinline__ PixWork prepare(const FrameArgs* frames, const int* i
   return w;
 }
 
+// Store, evict-first in L2 if `stream`.
+template <class T>
+__device__ __forceinline__ void put(T* p, T v, bool stream) {
+  if (stream) __stcs(p, v); else *p = v;
+}
+
 // Background (generation 0), then the K4 epilogue of one pixel: colour,
 // running sum (Kahan-compensated past the threshold), Welford M2, mean, RGBA8,
 // and one variance partial per warp of 32 pixels.  S, M, CP are the pixel's
 // previous sum, M2 and compensation.  Every lane of the warp calls it (the
 // partial is a warp reduction); inactive lanes contribute zero.
+template <int FR>
 __device__ __forceinline__ void finish_pixel(const FrameArgs* A, const PixWork& w, int lane,
                                              int warp, float c0, float c1, float c2, float al,
                                              bool covered, float4 S, float4 M, float4 CP,
@@ -718,7 +738,10 @@ __device__ __forceinline__ void finish_pixel(const FrameArgs* A, const PixWork& 
     const float4 col = make_float4(c0, c1, c2, al);
     const bool pixOk = DFB_CHECK(w.pix < (size_t)A->W * A->H, err);
     const bool stateOk = DFB_CHECK(w.sidx < (size_t)A->nTiles * A->T * A->T, err);
-    if ((flags & DFB_FLAG_WRITE_COLOR) && pixOk) A->color[w.pix] = col;
+    // images stream in frames that keep part of their state in L2
+    const bool stream = kKeeps<FR> && A->keepTiles != kKeepAll;
+    const bool streamState = kKeeps<FR> && w.tile >= A->keepTiles;
+    if ((flags & DFB_FLAG_WRITE_COLOR) && pixOk) put(A->color + w.pix, col, stream);
     float4 out = col;
     if (acc) {
       float4 Sn, tot;
@@ -734,7 +757,7 @@ __device__ __forceinline__ void finish_pixel(const FrameArgs* A, const PixWork& 
   }
         DFB_KAHAN(x) DFB_KAHAN(y) DFB_KAHAN(z) DFB_KAHAN(w)
 #undef DFB_KAHAN
-        if (stateOk) A->comp[w.sidx] = cn;
+        if (stateOk) put(A->comp + w.sidx, cn, streamState);
       } else {
         Sn = make_float4(S.x + col.x, S.y + col.y, S.z + col.z, S.w + col.w);
         tot = Sn;
@@ -749,14 +772,14 @@ __device__ __forceinline__ void finish_pixel(const FrameArgs* A, const PixWork& 
         M.w = fmaf(col.w - S.w * iN1, col.w - mean.w, M.w);
       }
       if (stateOk) {
-        A->accum[w.sidx] = Sn;
-        A->m2[w.sidx] = M;
+        put(A->accum + w.sidx, Sn, streamState);
+        put(A->m2 + w.sidx, M, streamState);
       }
       vsum = (M.x + M.y + M.z) * iN1;
       out = mean;
     }
     if ((flags & DFB_FLAG_PACK_RGBA8) && pixOk)
-      A->rgba8[w.pix] = pack_rgba8(pixel_op(out, A), tb);
+      put(A->rgba8 + w.pix, pack_rgba8(pixel_op(out, A), tb), stream);
   }
   if (acc && warp * 32 < w.P) {
     // one partial per warp of 32 pixels, summed per tile by k_tile_variance
@@ -857,6 +880,23 @@ __device__ __forceinline__ bool multi_fill(int total, const PixWork& w, int t, i
   return true;
 }
 
+// The pixel's state before this frame (the frame accumulates and is not the
+// first); FR's frames may choose what stays in L2.
+template <int FR>
+__device__ __forceinline__ void read_state(const FrameArgs* A, const PixWork& w, float4& S,
+                                           float4& M, float4& CP) {
+  const bool comp = A->kahan && !A->kahanFirst;
+  if (kKeeps<FR> && w.tile >= A->keepTiles) {
+    S = __ldcs(A->accum + w.sidx);
+    M = __ldcs(A->m2 + w.sidx);
+    if (comp) CP = __ldcs(A->comp + w.sidx);
+  } else {
+    S = A->accum[w.sidx];
+    M = A->m2[w.sidx];
+    if (comp) CP = A->comp[w.sidx];
+  }
+}
+
 // Consumer group: one pixel per thread.  Its items' fills come from its own
 // slots, in order.
 template <int DT, int G, int PER, int FR>
@@ -890,11 +930,8 @@ __device__ void consumer(const FrameArgs* __restrict__ frames, const int* __rest
     const PixWork v = prepare<FR>(frames, itemBase, 0, it, t);  // single-frame launches only
     const FrameArgs* B = v.A;
     if (v.active && (B->flags & DFB_FLAG_ACCUMULATE) && B->frameN != 1 && !B->stateInRing &&
-        DFB_CHECK(v.sidx < (size_t)B->nTiles * B->T * B->T, ctl.err)) {
-      s0 = B->accum[v.sidx];
-      m2 = B->m2[v.sidx];
-      if (B->kahan && !B->kahanFirst) cp = B->comp[v.sidx];
-    }
+        DFB_CHECK(v.sidx < (size_t)B->nTiles * B->T * B->T, ctl.err))
+      read_state<FR>(B, v, s0, m2, cp);
   };
   float4 nS0, nM, nCP;  // the next item's state (loads one item ahead)
   if constexpr (ahead) load_state(blockIdx.x, nS0, nM, nCP);
@@ -916,11 +953,7 @@ __device__ void consumer(const FrameArgs* __restrict__ frames, const int* __rest
       load_state(item + (int)gridDim.x, nS0, nM, nCP);
     } else {
       S0 = M = CP = zero4;
-      if (accRead && !A->stateInRing) {
-        S0 = A->accum[w.sidx];
-        M = A->m2[w.sidx];
-        if (A->kahan && !A->kahanFirst) CP = A->comp[w.sidx];
-      }
+      if (accRead && !A->stateInRing) read_state<FR>(A, w, S0, M, CP);
     }
     int s = group * S + jg % S;
     if (!wait_phase(&fullB[s], (uint32_t)(jg / S) & 1u, ctl, abort)) {
@@ -991,7 +1024,7 @@ __device__ void consumer(const FrameArgs* __restrict__ frames, const int* __rest
         continue;
       }
     }
-    finish_pixel(A, w, lane, warp, c0, c1, c2, al, covered, S0, M, CP, tb, ctl.err);
+    finish_pixel<FR>(A, w, lane, warp, c0, c1, c2, al, covered, S0, M, CP, tb, ctl.err);
   }
 }
 
@@ -1085,7 +1118,7 @@ __global__ void __launch_bounds__(kP, 2) k_composite_redo(const FrameArgs* __res
       M = A->m2[w.sidx];
       if (A->kahan && !A->kahanFirst) CP = A->comp[w.sidx];
     }
-    finish_pixel(A, w, lane, iw, c0, c1, c2, al, true, S, M, CP, tb, ctl.err);
+    finish_pixel<kGlobalTable>(A, w, lane, iw, c0, c1, c2, al, true, S, M, CP, tb, ctl.err);
   }
 }
 

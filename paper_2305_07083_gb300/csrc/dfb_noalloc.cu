@@ -280,6 +280,7 @@ int composite_noalloc(int width, int height, int tile_size, int mode, int dtype,
   a.flags = (color_out ? DFB_FLAG_WRITE_COLOR : 0u) | (rgba8_out ? DFB_FLAG_PACK_RGBA8 : 0u);
   a.frameN = 1;
   a.stateInRing = 0;  // no accumulation state
+  a.keepTiles = dfb::kKeepAll;
   a.invN = 1.0f;
   a.invNm1 = 0.0f;
   a.bgR = bg[0] * bg[3];
