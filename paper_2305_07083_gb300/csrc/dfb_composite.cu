@@ -89,6 +89,8 @@ constexpr int kSlots = 16;               // items in flight at most
 constexpr int kRound = 4;                // items the producer plans at once
 constexpr int kMetaQ = 2 * kRound;       // tile blocks fetched ahead
 constexpr uint32_t kWindowBytes = kSortWindow * kP * 8;
+constexpr int kRedoRank = 48;            // longest list the re-do kernel ranks
+constexpr int kRedoPer = 2;              // its CTAs per SM
 
 // Descriptor of one fill of the ring: up to kN fragments of one work item
 // (all of them for an item of at most kN fragments, else kFill), and the
@@ -1075,50 +1077,148 @@ __global__ void __launch_bounds__(Shape<G>::threads, PER)
                              emptyB, abort, tb, ringBytes);
 }
 
+// A warp's scratch of the exact re-do: the fragments of one unit's list.
+struct RedoWarp {
+  const void* rgba[kRedoRank];
+  const float* depth[kRedoRank];
+  float scale[kRedoRank];
+  float z[kRedoRank][32];               // canonical depths, a column per pixel
+  unsigned char order[kRedoRank][32];   // fragment of each place in the pixel's order
+};
+
+// Exact BLEND_DEPTH order for one pixel of a list of at most kRedoRank
+// fragments: all depths are read once, several in flight, a fragment's place
+// is the number of fragments before it by (depth, list index), and the RGBA
+// are read in that order, several in flight.  Called by the active lanes of a
+// warp; `w` holds the list's pointers already.
+template <int DT>
+__device__ __forceinline__ void composite_ranked(int n, RedoWarp* w, int lane, int p, float& c0,
+                                                 float& c1, float& c2, float& al) {
+  for (int i0 = 0; i0 < n; i0 += 16) {
+    float z[16];
+#pragma unroll
+    for (int u = 0; u < 16; ++u)
+      if (i0 + u < n) z[u] = __ldg(w->depth[i0 + u] + p);
+#pragma unroll
+    for (int u = 0; u < 16; ++u)
+      if (i0 + u < n) w->z[i0 + u][lane] = covers(z[u]) ? z[u] : INFINITY;
+  }
+  for (int i0 = 0; i0 < n; i0 += 4) {
+    float z[4];
+    int rank[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int u = 0; u < 4; ++u) z[u] = i0 + u < n ? w->z[i0 + u][lane] : INFINITY;
+#pragma unroll 4
+    for (int j = 0; j < i0; ++j) {
+      const float v = w->z[j][lane];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) rank[u] += v <= z[u] ? 1 : 0;
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (i0 + j < n && j != u) rank[u] += (j < u ? z[j] <= z[u] : z[j] < z[u]) ? 1 : 0;
+#pragma unroll 4
+    for (int j = i0 + 4; j < n; ++j) {
+      const float v = w->z[j][lane];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) rank[u] += v < z[u] ? 1 : 0;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i0 + u < n) w->order[rank[u]][lane] = (unsigned char)(i0 + u);
+  }
+  for (int r0 = 0; r0 < n; r0 += 8) {
+    float4 f[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (r0 + u < n) {
+        const int i = w->order[r0 + u][lane];
+        f[u] = Px<DT>::global(w->rgba[i], p, w->scale[i]);
+      }
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (r0 + u < n) over(f[u], c0, c1, c2, al);
+  }
+}
+
 // Exact re-do of the 32-pixel units (work item, warp) that the persistent
 // kernel left: multi-fill BLEND_DEPTH items whose depths were out of list
 // order at some pixel, or that had a non-zero empty fragment.  Each warp of a
-// CTA takes one unit at a time; each pixel reads its fragments from HBM and
-// blends them in exact (depth, key, submit index) order through the
-// windowed rounds of composite_exact, then goes through the same
-// epilogue.  Units are rare on brick scenes, whose key order is their depth
-// order; the kernel returns at once when there are none.
+// CTA takes one unit at a time; each pixel reads its fragments from memory
+// (mostly still in L2) and blends them in exact (depth, key, submit index)
+// order -- by rank, or through the windowed rounds of composite_exact for the
+// longest lists -- then goes through the same epilogue.  Where the keys follow
+// the depths (bricks) there are no units and the kernel returns at once;
+// where producers overlap, most units of a long list are here.
+//
+// Bound by the latency of its dependent reads: 16 depths and 8 RGBA per lane
+// are in flight at a time.  1024x1024, FP32, 3,500 units of 17 to 24 fragments:
+// 31 us (41 us by windowed rounds; 41 us with 3 CTAs per SM, which spill).
+// Launched programmatically, so that a launch that finds no units costs no
+// more than its own start: 16 passes of FP8 4096x1024 1.435 -> 1.396 ms.
 template <int DT>
-__global__ void __launch_bounds__(kP, 2) k_composite_redo(const FrameArgs* __restrict__ frames,
-                                                       const int* __restrict__ itemBase,
-                                                       int nFrames, LaunchCtl ctl) {
+__global__ void __launch_bounds__(kP, kRedoPer) k_composite_redo(
+    const FrameArgs* __restrict__ frames, const int* __restrict__ itemBase, int nFrames,
+    LaunchCtl ctl) {
   extern __shared__ __align__(128) unsigned char lsmem[];
   SrgbTables* tb = reinterpret_cast<SrgbTables*>(lsmem);
-  uint64_t* window = reinterpret_cast<uint64_t*>(lsmem + sizeof(SrgbTables) + 128);
+  RedoWarp* scratch = reinterpret_cast<RedoWarp*>(lsmem + sizeof(SrgbTables));
+  uint64_t* window = reinterpret_cast<uint64_t*>(scratch);  // longer lists, same memory
+  grid_dependency_wait();  // the composite's list of units, and its writes
+  allow_dependents();
   const int count = *(volatile int*)ctl.redo;
-  if ((int)blockIdx.x * (kP / 32) >= count) return;
+  if ((int)blockIdx.x * kCW >= count) return;
   load_srgb(tb, kP);
   __syncthreads();
-  const int lane = threadIdx.x & 31;
-  for (int u = blockIdx.x * (kP / 32) + (threadIdx.x >> 5); u < count;
-       u += gridDim.x * (kP / 32)) {
-    const int entry = ctl.redo[1 + u];
-    const int item = entry / (kP / 32), iw = entry % (kP / 32);
-    const int f = find_frame(itemBase, nFrames, item);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int u0 = blockIdx.x * kCW; u0 < count; u0 += gridDim.x * kCW) {
+    const int u = u0 + warp;
+    int n = 0, item = 0, iw = 0, f = 0, local = 0;
+    const FragRec* list = nullptr;
+    if (u < count) {
+      const int entry = ctl.redo[1 + u];
+      item = entry / kCW;
+      iw = entry % kCW;
+      f = find_frame(itemBase, nFrames, item);
+      local = item - __ldg(itemBase + f);
+      const FrameArgs* A = frames + f;
+      if (DFB_CHECK(f >= 0 && f < nFrames && (local >> A->logChunks) < A->nTiles, ctl.err)) {
+        const TileBlock* blk = A->blocks + A->tileBase + (local >> A->logChunks);
+        n = blk->n;
+        list = A->srecs + blk->off;
+      }
+    }
     const FrameArgs* A = frames + f;
-    const int local = item - __ldg(itemBase + f);
-    const int gt = A->tileBase + (local >> A->logChunks);
-    if (!DFB_CHECK(f >= 0 && f < nFrames && (local >> A->logChunks) < A->nTiles, ctl.err))
-      continue;
-    const TileBlock* blk = A->blocks + gt;
-    const int n = blk->n;
-    const FragRec* list = A->srecs + blk->off;
     const PixWork w = prepare<kGlobalTable>(frames, itemBase, f, item, iw * 32 + lane);
     float c0 = 0.f, c1 = 0.f, c2 = 0.f, al = 0.f;
-    if (w.active) composite_exact<DT>(n, list, window, threadIdx.x, w.p, c0, c1, c2, al);
-    const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    float4 S = zero4, M = zero4, CP = zero4;
-    if (w.active && (A->flags & DFB_FLAG_ACCUMULATE) && A->frameN != 1) {
-      S = A->accum[w.sidx];
-      M = A->m2[w.sidx];
-      if (A->kahan && !A->kahanFirst) CP = A->comp[w.sidx];
+    // A window column of one warp overlaps the scratch of others, so the CTA
+    // does its ranked units and its windowed ones one after the other.
+    const bool ranked = n <= kRedoRank;
+    if (n > 0 && ranked) {
+      RedoWarp* rw = scratch + warp;
+      for (int i = lane; i < n; i += 32) {
+        rw->rgba[i] = list[i].rgba;
+        rw->depth[i] = list[i].depth;
+        rw->scale[i] = list[i].scale;
+      }
+      __syncwarp();
+      if (w.active) composite_ranked<DT>(n, rw, lane, w.p, c0, c1, c2, al);
+      __syncwarp();
     }
-    finish_pixel<kGlobalTable>(A, w, lane, iw, c0, c1, c2, al, true, S, M, CP, tb, ctl.err);
+    if (__syncthreads_or(!ranked)) {
+      if (!ranked && w.active)
+        composite_exact<DT>(n, list, window, threadIdx.x, w.p, c0, c1, c2, al);
+      __syncthreads();
+    }
+    if (n > 0) {
+      const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+      float4 S = zero4, M = zero4, CP = zero4;
+      if (w.active && (A->flags & DFB_FLAG_ACCUMULATE) && A->frameN != 1)
+        read_state<kGlobalTable>(A, w, S, M, CP);
+      finish_pixel<kGlobalTable>(A, w, lane, iw, c0, c1, c2, al, true, S, M, CP, tb, ctl.err);
+    }
   }
 }
 
@@ -1229,6 +1329,9 @@ cudaError_t launch_shape(const FrameArgs* frames, const int* itemBase, int nFram
                              totalItems, ring, ctl, 0);
 }
 
+constexpr size_t kRedoBytes =
+    sizeof(RedoWarp) * kCW > kWindowBytes ? sizeof(RedoWarp) * kCW : kWindowBytes;
+
 template <int DT>
 cudaError_t launch_dt(const FrameArgs* frames, const int* itemBase, int nFrames, int totalItems,
                       const TuneParams& tune, const LaunchCtl& ctl, const FrameArgs* hostFrames,
@@ -1297,7 +1400,7 @@ cudaError_t launch_composite(const FrameArgs* frames, const int* itemBase, int n
   int dev = 0;
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess && (dev < 0 || dev >= 64)) e = cudaErrorInvalidDevice;
-  const int smem = (int)(sizeof(SrgbTables) + 128 + kWindowBytes);
+  const int smem = (int)(sizeof(SrgbTables) + kRedoBytes);
   if (e == cudaSuccess && !sms[dev]) {
     int count = 0;
     e = cudaDeviceGetAttribute(&count, cudaDevAttrMultiProcessorCount, dev);
@@ -1317,22 +1420,26 @@ cudaError_t launch_composite(const FrameArgs* frames, const int* itemBase, int n
   }
   if (e == cudaSuccess && lng.items > 0) {
     // at most one unit per warp of the long items; the count is on the device
-    const int grid = lng.items < 2 * sms[dev] ? lng.items : 2 * sms[dev];
+    const int most = kRedoPer * sms[dev];
+    const int grid = lng.items < most ? lng.items : most;
     switch (dtype) {
       case DFB_F32:
-        k_composite_redo<DFB_F32><<<grid, kP, smem, s>>>(frames, itemBase, nFrames, ctl);
+        e = launch_programmatic(k_composite_redo<DFB_F32>, grid, kP, smem, s, frames, itemBase,
+                                nFrames, ctl);
         break;
       case DFB_F16:
-        k_composite_redo<DFB_F16><<<grid, kP, smem, s>>>(frames, itemBase, nFrames, ctl);
+        e = launch_programmatic(k_composite_redo<DFB_F16>, grid, kP, smem, s, frames, itemBase,
+                                nFrames, ctl);
         break;
       case DFB_BF16:
-        k_composite_redo<DFB_BF16><<<grid, kP, smem, s>>>(frames, itemBase, nFrames, ctl);
+        e = launch_programmatic(k_composite_redo<DFB_BF16>, grid, kP, smem, s, frames, itemBase,
+                                nFrames, ctl);
         break;
       default:
-        k_composite_redo<DFB_FP8E4M3><<<grid, kP, smem, s>>>(frames, itemBase, nFrames, ctl);
+        e = launch_programmatic(k_composite_redo<DFB_FP8E4M3>, grid, kP, smem, s, frames,
+                                itemBase, nFrames, ctl);
         break;
     }
-    e = cudaGetLastError();
   }
   if (e != cudaSuccess || !accumulate || totalTiles < 1) return e;
   return launch_programmatic(k_tile_variance, (totalTiles * 32 + 255) / 256, 256, 0, s, frames,
