@@ -555,6 +555,7 @@ __device__ __forceinline__ bool composite_staged(int mode, int n, int P, const u
   // floats per depth slab (no depth is staged in the modes that ignore it)
   const int dStride = mode == DFB_BLEND_DEPTH || mode == DFB_ZCOMPOSITE ? P : 0;
   const unsigned char* sC = base + (size_t)n * dStride * 4;
+  const int stride = FULL ? kP : P;
   if (mode == DFB_BLEND_ORDERED) {
     blend_list<DT, DFB_BLEND_ORDERED, FULL>(n, P, sC, meta, t, c0, c1, c2, al);
   } else if (mode == DFB_AVERAGE) {
@@ -583,31 +584,32 @@ __device__ __forceinline__ bool composite_staged(int mode, int n, int P, const u
       if (!bad && rest == 0u) return true;
       c0 = c1 = c2 = al = 0.0f;
     }
-    // General case: insertion sort of fragment indices (4-bit slots of
-    // `perm`) by depth key.  The list arrives in key order, so ties stay in
-    // (key, submit index) order; empty fragments go to a second list kept in
-    // list order and blended last.
+    // General case: sort of fragment indices (4-bit slots of `perm`) by
+    // depth.  The list arrives in key order, so ties stay in (key, submit
+    // index) order; empty fragments go to a second list kept in list order
+    // and blended last.  A finite fragment goes in front of the finite ones
+    // before it in the list that are deeper: they are counted, over all of
+    // the list so far, by loads that do not depend on one another (empty
+    // ones do not count).
+    const float* zt = sD + t;
     uint64_t perm = 0, infs = 0;
     int m = 0, mi = 0;
-    uint32_t lastKey = 0;
     for (int i = 0; i < n; ++i) {
-      const uint32_t key = depth_bits(sD[i * P + t]);
-      const bool isInf = key == kInfBits;
-      const bool app = !isInf && (m == 0 || key >= lastKey);
-      if (!isInf && !app) {
-        int j = m - 1;
-        while (j > 0 && depth_bits(sD[(int)((perm >> (4 * (j - 1))) & 15u) * P + t]) > key) --j;
-        const uint64_t lowMask = (j == 0) ? 0ull : ((1ull << (4 * j)) - 1ull);
-        perm = (perm & lowMask) | ((uint64_t)i << (4 * j)) | ((perm & ~lowMask) << 4);
-        ++m;
+      const float z = zt[i * stride];
+      const bool in = covers(z);
+      int deeper = 0;
+#pragma unroll 4
+      for (int j = 0; j < i; ++j) {
+        const float v = zt[j * stride];
+        deeper += covers(v) && v > z ? 1 : 0;
       }
-      // appends to either list without a branch
-      const uint64_t bit = (uint64_t)i << (4 * (isInf ? mi : m));
-      infs |= isInf ? bit : 0ull;
-      perm |= app ? bit : 0ull;
-      lastKey = app ? key : lastKey;
-      mi += isInf ? 1 : 0;
-      m += app ? 1 : 0;
+      const int at = 4 * (m - deeper);
+      const uint64_t low = perm & ((1ull << at) - 1ull);
+      const uint64_t put = low | ((uint64_t)i << at) | ((perm ^ low) << 4);
+      perm = in ? put : perm;
+      infs |= in ? 0ull : (uint64_t)i << (4 * mi);
+      m += in ? 1 : 0;
+      mi += in ? 0 : 1;
     }
     // one loop of exactly n steps: the finite list, then the empty ones
     for (int r = 0; r < n; ++r) {
