@@ -24,13 +24,10 @@ cudaError_t upload_srgb_tables(const SrgbTables& host);
 using dfb::FragRec;
 using dfb::FrameArgs;
 
-// What one frame uploads ahead of its records: the frame's arguments and the
-// work-item prefix of a one-frame launch.  A multiple of 32 bytes so the
-// records that follow stay aligned.
-struct FrameHeader {
-  FrameArgs fa;
-  int itemBase[2];
-};
+using dfb::FrameHeader;
+
+// A frame's upload starts with its header, padded to a multiple of 32 bytes
+// so that the records that follow stay aligned.
 constexpr size_t kHdrBytes = (sizeof(FrameHeader) + 31) / 32 * 32;
 
 namespace {
@@ -172,7 +169,10 @@ struct dfb_ctx {
   int arenaIdx = 0;
   cudaStream_t copyStream = nullptr;
   cudaEvent_t copyDone = nullptr;
-  cudaEvent_t frameDone = nullptr;
+  cudaEvent_t frameDone = nullptr;  // end of a frame of a batch or graph
+  // Recorded behind the handle's last frame: frameDone, or the `released` of
+  // the set that the frame used.
+  cudaEvent_t done = nullptr;
   cudaStream_t lastStream = nullptr;
   bool lastStreamSet = false;
 
@@ -276,7 +276,7 @@ int grow_records(dfb_ctx* h, size_t need) {
   while (cap < need) cap *= 2;
   // Earlier frames may still read the old arrays (the last frame's
   // composite is ordered after every earlier bucketing and composite).
-  if (h->lastStreamSet) cudaEventSynchronize(h->frameDone);
+  if (h->lastStreamSet) cudaEventSynchronize(h->done);
   h->recCap = 0;
   for (BucketSet& b : h->sets) {
     cudaFree(b.dStage);
@@ -352,7 +352,7 @@ void free_device(dfb_ctx* h) {
   if (h->copyDone) cudaEventDestroy(h->copyDone);
   if (h->frameDone) cudaEventDestroy(h->frameDone);
   h->copyStream = nullptr;
-  h->copyDone = h->frameDone = nullptr;
+  h->copyDone = h->frameDone = h->done = nullptr;
   h->allocated = false;
 }
 
@@ -831,7 +831,7 @@ int dfb_create(int width, int height, int tile_size, int mode, dfb_handle* out) 
 int dfb_destroy(dfb_handle h) {
   return guarded([&]() -> int {
     if (!h) return DFB_OK;
-    if (h->allocated && h->lastStreamSet) cudaEventSynchronize(h->frameDone);
+    if (h->allocated && h->lastStreamSet) cudaEventSynchronize(h->done);
     free_device(h);
     if (h->curve) cudaFree(h->curve);
     delete h;
@@ -880,7 +880,7 @@ int dfb_set_pixel_curve(dfb_handle h, const float* curves, int n, float x_max) {
       h->curveDevice = dev;
     } else if (h->allocated && h->lastStreamSet) {
       // frames in flight may still read the previous samples
-      e = cudaEventSynchronize(h->frameDone);
+      e = cudaEventSynchronize(h->done);
       if (e != cudaSuccess) return DFB_ERR_CUDA;
     }
     // the legacy stream, waited for: the DMA of a pageable source has landed
@@ -1154,55 +1154,74 @@ int take_device_error(dfb_ctx* h) {
 }
 
 int end_one(dfb_ctx* h, cudaStream_t s) {
-  FragRec* staged = nullptr;
-  int st = grow_records(h, h->recs.size());
+  const size_t n = h->recs.size();
+  int st = grow_records(h, n);
   if (st != DFB_OK) return st;
-  const int buf = stage_records(h, &staged);
+  // A frame whose records fit a kernel parameter needs no upload and no side
+  // stream: its bucketing is a launch on `s` (256x256, 8 bricks: the pass takes
+  // 27 to 30 us instead of 36).  Few records of large tiles are left to the side stream:
+  // from about a million pixels the composite takes longer than the host, and
+  // a bucketing beside the previous composite costs nothing.
+  const size_t mostPixels = (size_t)1 << 20;
+  const bool small = n <= (size_t)dfb::kInlineRecs && h->nTiles <= dfb::kInlineTiles &&
+                     (n + (size_t)h->nTiles) * h->tilePixels <= mostPixels;
+  dfb::InlineFrame in;
+  FragRec* staged = nullptr;
+  const int buf = small ? 0 : stage_records(h, &staged);
   if (buf < 0) return buf;
   BucketSet& b = h->sets[h->setIdx];
   h->setIdx ^= 1;
-  const size_t n = h->recs.size();
   // header: the frame's arguments + the item prefix of a one-frame launch
-  FrameHeader* hdr = reinterpret_cast<FrameHeader*>(staged);
+  FrameHeader* hdr = small ? &in.hdr : reinterpret_cast<FrameHeader*>(staged);
   fill_frame_args(h, hdr->fa, 0, b.srecs, b.blocks);
   hdr->itemBase[0] = 0;
   hdr->itemBase[1] = h->nTiles * hdr->fa.chunks;
   const int items = hdr->itemBase[1];
-  FrameArgs* dFa = reinterpret_cast<FrameArgs*>(b.dStage);
-  const int* dItemBase = reinterpret_cast<const int*>(b.dStage + offsetof(FrameHeader, itemBase));
-  const int* dTileOff = reinterpret_cast<const int*>(b.dStage + kHdrBytes + sizeof(FragRec) * n);
+  FrameHeader* dHdr = reinterpret_cast<FrameHeader*>(b.dStage);
   // only BLEND_DEPTH items can need the exact re-do kernel
   const int nLong = h->cfg.mode == DFB_BLEND_DEPTH ? (int)h->longTiles.size() : 0;
   dfb::LongList lng;
   lng.items = nLong * h->chunks;
   for (int t : h->longTiles) lng.maxFragments = std::max(lng.maxFragments, h->fragCount[t]);
-  // The bucketing reads only library-owned buffers, so it runs on the side
-  // stream, overlapping the previous frame's composite (dfb_end_frames has
-  // refused a capturing stream).
   cudaError_t e = cudaSuccess;
-  cudaStream_t bs = h->bucketStream;
-  if (h->lastStreamSet && h->lastStream != s) e = cudaStreamWaitEvent(s, h->frameDone, 0);
-  if (e == cudaSuccess && b.used) e = cudaStreamWaitEvent(bs, b.released, 0);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(b.dStage, staged, stage_bytes(h, n), cudaMemcpyHostToDevice, bs);
-  if (e == cudaSuccess) e = cudaEventRecord(h->hRecDone[buf], bs);
+  if (h->lastStreamSet && h->lastStream != s) e = cudaStreamWaitEvent(s, h->done, 0);
   cudaEvent_t* ev = timing_slot(h);
-  if (e == cudaSuccess && ev) e = cudaEventRecord(ev[0], bs);
-  if (e == cudaSuccess)
-    e = dfb::launch_bucket(b.dRecs, dTileOff, h->nTiles, b.srecs, b.blocks, b.redo, bs);
-  if (e == cudaSuccess && ev) e = cudaEventRecord(ev[1], bs);
-  if (e == cudaSuccess) e = cudaEventRecord(b.ready, bs);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(s, b.ready, 0);
+  if (small) {
+    // ordered behind everything that used the set: the composite that read it
+    // last is behind `done`, and so is the bucketing it waited for
+    in.nTiles = h->nTiles;
+    group_by_tile(h->recs.data(), n, h->fragCount.data(), h->nTiles, 0, in.recs, in.tileOff,
+                  h->tileCursor);
+    if (e == cudaSuccess && ev) e = cudaEventRecord(ev[0], s);
+    if (e == cudaSuccess) e = dfb::launch_bucket_inline(in, dHdr, b.srecs, b.blocks, b.redo, s);
+    if (e == cudaSuccess && ev) e = cudaEventRecord(ev[1], s);
+  } else {
+    // The bucketing reads only library-owned buffers, so it runs on the side
+    // stream, overlapping the previous frame's composite (dfb_end_frames has
+    // refused a capturing stream).
+    cudaStream_t bs = h->bucketStream;
+    const int* dTileOff = reinterpret_cast<const int*>(b.dStage + kHdrBytes + sizeof(FragRec) * n);
+    if (e == cudaSuccess && b.used) e = cudaStreamWaitEvent(bs, b.released, 0);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(b.dStage, staged, stage_bytes(h, n), cudaMemcpyHostToDevice, bs);
+    if (e == cudaSuccess) e = cudaEventRecord(h->hRecDone[buf], bs);
+    if (e == cudaSuccess && ev) e = cudaEventRecord(ev[0], bs);
+    if (e == cudaSuccess)
+      e = dfb::launch_bucket(b.dRecs, dTileOff, h->nTiles, b.srecs, b.blocks, b.redo, bs);
+    if (e == cudaSuccess && ev) e = cudaEventRecord(ev[1], bs);
+    if (e == cudaSuccess) e = cudaEventRecord(b.ready, bs);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, b.ready, 0);
+  }
   if (e == cudaSuccess && h->hostCopies) e = cudaStreamWaitEvent(s, h->copyDone, 0);
   if (e == cudaSuccess && ev) e = cudaEventRecord(ev[2], s);
   if (e == cudaSuccess)
-    e = dfb::launch_composite(dFa, dItemBase, 1, items, h->nTiles,
+    e = dfb::launch_composite(&dHdr->fa, dHdr->itemBase, 1, items, h->nTiles,
                               (h->cfg.flags & DFB_FLAG_ACCUMULATE) != 0, h->cfg.dtype,
                               tune_of(h, n, (size_t)h->nTiles, true),
                               ctl_of(h, b.redo), lng, &hdr->fa, hdr->itemBase,
                               ev ? ev[3] : nullptr, s);
   if (e == cudaSuccess) e = cudaEventRecord(b.released, s);
-  if (e == cudaSuccess) e = cudaEventRecord(h->frameDone, s);
+  if (e == cudaSuccess) h->done = b.released;
   b.used = true;
   h->launches += 1 + ((h->cfg.flags & DFB_FLAG_ACCUMULATE) ? 2 : 1) + (nLong ? 1 : 0);
   h->lastErr = h->errFlag;
@@ -1268,7 +1287,7 @@ int end_batch(dfb_ctx* const* hs, int n, cudaStream_t s) {
     items += h->nTiles * b.hFrames[i].chunks;
     tileBase += h->nTiles;
     if (h->lastStreamSet && h->lastStream != s && e == cudaSuccess)
-      e = cudaStreamWaitEvent(s, h->frameDone, 0);
+      e = cudaStreamWaitEvent(s, h->done, 0);
     if (h->hostCopies && e == cudaSuccess) e = cudaStreamWaitEvent(s, h->copyDone, 0);
   }
   b.hItemBase[n] = items;
@@ -1304,6 +1323,7 @@ int end_batch(dfb_ctx* const* hs, int n, cudaStream_t s) {
   hs[0]->stallItem = -1;
   for (int i = 0; i < n && e == cudaSuccess; ++i) {
     e = cudaEventRecord(hs[i]->frameDone, s);
+    hs[i]->done = hs[i]->frameDone;
     hs[i]->lastErr = hs[0]->errFlag;
   }
   return cuda_status(e);
@@ -1363,7 +1383,7 @@ int dfb_sync(dfb_handle h) {
   return guarded([&]() -> int {
     if (!h) return DFB_ERR_INVALID_ARG;
     if (!h->lastStreamSet) return DFB_OK;
-    const int st = cuda_status(cudaEventSynchronize(h->frameDone));
+    const int st = cuda_status(cudaEventSynchronize(h->done));
     return st != DFB_OK ? st : take_device_error(h);
   });
 }
@@ -1799,7 +1819,7 @@ int dfb_graph_create(const dfb_handle* hs, int n, dfb_graph* out) {
     for (int i = 0; i < n; ++i) {
       const int st = allocate(hs[i]);
       if (st != DFB_OK) return st;
-      if (hs[i]->lastStreamSet) cudaEventSynchronize(hs[i]->frameDone);
+      if (hs[i]->lastStreamSet) cudaEventSynchronize(hs[i]->done);
       if (hs[i]->hostCopies) cudaEventSynchronize(hs[i]->copyDone);
     }
     dfb_graph_t* g = new (std::nothrow) dfb_graph_t();
@@ -1822,6 +1842,7 @@ int dfb_graph_launch(dfb_graph g, void* stream) {
     for (size_t i = 0; i < g->hs.size() && e == cudaSuccess; ++i) {
       dfb_ctx* h = g->hs[i];
       e = cudaEventRecord(h->frameDone, s);
+      h->done = h->frameDone;
       h->lastStream = s;
       h->lastStreamSet = true;
       h->haveFrame = true;

@@ -50,8 +50,6 @@
 // drains its own bulk copies and returns.
 #include <string.h>
 
-#include <utility>
-
 #include "dfb_device.cuh"
 #include "dfb_internal.h"
 
@@ -1254,25 +1252,6 @@ __global__ void k_tile_variance(const FrameArgs* __restrict__ frames, int nFrame
     const int w = min(T, A->W - tx * T), h = min(T, A->H - ty * T);
     A->tileVar[tile] = sum / (3.0f * (float)(w * h));
   }
-}
-
-// Launch with programmatic stream serialisation: the kernel's blocks may be
-// scheduled before the previous kernel in the stream has finished; the
-// kernel's grid_dependency_wait() keeps its dependent accesses after it.
-template <typename... Params, typename... Args>
-cudaError_t launch_programmatic(void (*kernel)(Params...), int grid, int threads, size_t smem,
-                                cudaStream_t s, Args&&... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
 template <int DT, int G, int PER>

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
+
 #include "../../include/dfb.h"
 
 namespace dfb {
@@ -100,6 +102,24 @@ struct FrameArgs {
   const float* curve;          // DFB_PIXELOP_CURVE: 3 * curveN samples, channel-major
 };
 
+// What one frame uploads ahead of its records: the frame's arguments and the
+// work-item prefix of a one-frame launch.
+struct FrameHeader {
+  FrameArgs fa;
+  int itemBase[2];
+};
+
+// A frame small enough to travel as a kernel parameter: its header, the
+// offsets of its tiles' lists and its records grouped by tile.
+constexpr int kInlineTiles = 128;
+constexpr int kInlineRecs = 128;
+struct InlineFrame {
+  FrameHeader hdr;
+  int nTiles;
+  int tileOff[kInlineTiles + 1];
+  FragRec recs[kInlineRecs];
+};
+
 // Samples per channel of a user tone curve (DFB_PIXELOP_CURVE), at most.
 constexpr int kMaxCurve = 4096;
 
@@ -162,6 +182,12 @@ struct LaunchCtl {
 cudaError_t launch_bucket(const FragRec* grouped, const int* tileOff, int nTiles, FragRec* srecs,
                           TileBlock* blocks, int* redo, cudaStream_t s);
 
+// The same for a frame passed by value: no upload, and on the stream of the
+// composite that follows (launched programmatically), which also reads
+// `hdr`, the device copy of the frame's header written here.
+cudaError_t launch_bucket_inline(const InlineFrame& frame, FrameHeader* hdr, FragRec* srecs,
+                                 TileBlock* blocks, int* redo, cudaStream_t s);
+
 // Composite + accumulate + variance + pack (K2/K3 + K4) over the work items of
 // `nFrames` frames (device arrays `frames` and `itemBase`, nFrames + 1 prefix
 // of work items), all of storage dtype `dtype`, one persistent launch; then,
@@ -199,6 +225,25 @@ cudaError_t launch_image_to_tiles(const float4* in, float4* out, int W, int H, i
 // FP32 -> storage dtype conversion of fragment tiles (producer side).
 cudaError_t launch_convert(const float* src, void* dst, float* scales, int nTiles,
                            int tilePixels, int dtype, cudaStream_t s);
+
+// Launch with programmatic stream serialisation: the kernel's blocks may be
+// scheduled before the previous kernel in the stream has finished; the
+// kernel's grid_dependency_wait() keeps its dependent accesses after it.
+template <typename... Params, typename... Args>
+cudaError_t launch_programmatic(void (*kernel)(Params...), int grid, int threads, size_t smem,
+                                cudaStream_t s, Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
 
 // Upload the sRGB threshold table to the current device (idempotent).
 cudaError_t ensure_tables();

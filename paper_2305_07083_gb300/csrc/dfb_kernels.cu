@@ -9,6 +9,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include "dfb_device.cuh"
 #include "dfb_internal.h"
 
 namespace dfb {
@@ -26,18 +27,11 @@ constexpr int kSortSmem = 256;
 // final place is its rank under that key: the (key, submit index) order.
 // Lists of up to 32 are ranked in registers, longer ones sorted in shared
 // memory.
-__global__ void __launch_bounds__(kOrderWarps * 32) k1_order(const FragRec* __restrict__ grouped,
-                                                            const int* __restrict__ tileOff,
-                                                            int nTiles, FragRec* __restrict__ srecs,
-                                                            TileBlock* __restrict__ blocks,
-                                                            int* __restrict__ redo) {
-  __shared__ uint64_t keys[kOrderWarps][kSortSmem];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int t = blockIdx.x * kOrderWarps + warp;
-  if (redo && blockIdx.x == 0 && threadIdx.x == 0) redo[0] = 0;
-  if (t >= nTiles) return;
-  const int off = __ldg(tileOff + t);
-  const int n = __ldg(tileOff + t + 1) - off;
+__device__ __forceinline__ void order_tile(const FragRec* grouped, const int* tileOff, int t,
+                                           FragRec* __restrict__ srecs,
+                                           TileBlock* __restrict__ blocks, uint64_t* a, int lane) {
+  const int off = tileOff[t];
+  const int n = tileOff[t + 1] - off;
   if (lane == 0) {
     blocks[t].n = n;
     blocks[t].off = off;
@@ -59,11 +53,10 @@ __global__ void __launch_bounds__(kOrderWarps * 32) k1_order(const FragRec* __re
     return;
   }
   if (n <= kSortSmem) {
-    uint64_t* a = keys[warp];
     int m = 64;
     while (m < n) m <<= 1;
     for (int i = lane; i < m; i += 32)
-      a[i] = i < n ? (((uint64_t)__ldg(&in[i].key) << 32) | (uint32_t)i) : ~0ull;
+      a[i] = i < n ? (((uint64_t)in[i].key << 32) | (uint32_t)i) : ~0ull;
     __syncwarp();
     for (int k = 2; k <= m; k <<= 1) {
       for (int j = k >> 1; j > 0; j >>= 1) {
@@ -91,11 +84,11 @@ __global__ void __launch_bounds__(kOrderWarps * 32) k1_order(const FragRec* __re
   // very long lists: rank of each element by counting the smaller keys
   for (int jb = 0; jb < n; jb += 32) {
     const int j = jb + lane;
-    const uint64_t kj = j < n ? (((uint64_t)__ldg(&in[j].key) << 32) | (uint32_t)j) : ~0ull;
+    const uint64_t kj = j < n ? (((uint64_t)in[j].key << 32) | (uint32_t)j) : ~0ull;
     int rank = 0;
     for (int mb = 0; mb < n; mb += 32) {
       const int m = mb + lane;
-      const uint64_t km = m < n ? (((uint64_t)__ldg(&in[m].key) << 32) | (uint32_t)m) : ~0ull;
+      const uint64_t km = m < n ? (((uint64_t)in[m].key << 32) | (uint32_t)m) : ~0ull;
       const int cnt = min(32, n - mb);
       for (int q = 0; q < cnt; ++q) rank += (__shfl_sync(0xffffffffu, km, q) < kj) ? 1 : 0;
     }
@@ -107,11 +100,54 @@ __global__ void __launch_bounds__(kOrderWarps * 32) k1_order(const FragRec* __re
   }
 }
 
+__global__ void __launch_bounds__(kOrderWarps * 32) k1_order(const FragRec* __restrict__ grouped,
+                                                            const int* __restrict__ tileOff,
+                                                            int nTiles, FragRec* __restrict__ srecs,
+                                                            TileBlock* __restrict__ blocks,
+                                                            int* __restrict__ redo) {
+  __shared__ uint64_t keys[kOrderWarps][kSortSmem];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int t = blockIdx.x * kOrderWarps + warp;
+  if (redo && blockIdx.x == 0 && threadIdx.x == 0) redo[0] = 0;
+  if (t < nTiles) order_tile(grouped, tileOff, t, srecs, blocks, keys[warp], lane);
+}
+
+// A small frame's records come with the launch itself.  An upload, a launch
+// on a side stream and the events between the streams cost the host more
+// than such a frame takes on the GPU; here the bucketing is one more launch
+// on the frame's own stream.
+__global__ void __launch_bounds__(kOrderWarps * 32)
+    k1_order_inline(const __grid_constant__ InlineFrame frame, FrameHeader* __restrict__ hdr,
+                    FragRec* __restrict__ srecs, TileBlock* __restrict__ blocks,
+                    int* __restrict__ redo) {
+  __shared__ uint64_t keys[kOrderWarps][kSortSmem];
+  grid_dependency_wait();  // an earlier frame may still read the buffers
+  allow_dependents();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int t = blockIdx.x * kOrderWarps + warp;
+  if (blockIdx.x == 0) {
+    if (redo && threadIdx.x == 0) redo[0] = 0;
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(&frame.hdr);
+    for (int i = threadIdx.x; i < (int)(sizeof(FrameHeader) / 4); i += kOrderWarps * 32)
+      reinterpret_cast<uint32_t*>(hdr)[i] = src[i];
+  }
+  if (t < frame.nTiles)
+    order_tile(frame.recs, frame.tileOff, t, srecs, blocks, keys[warp], lane);
+}
+
 cudaError_t launch_bucket(const FragRec* grouped, const int* tileOff, int nTiles, FragRec* srecs,
                           TileBlock* blocks, int* redo, cudaStream_t s) {
   const int grid = nTiles > 0 ? (nTiles + kOrderWarps - 1) / kOrderWarps : 1;
   k1_order<<<grid, kOrderWarps * 32, 0, s>>>(grouped, tileOff, nTiles, srecs, blocks, redo);
   return cudaGetLastError();
+}
+
+cudaError_t launch_bucket_inline(const InlineFrame& frame, FrameHeader* hdr, FragRec* srecs,
+                                 TileBlock* blocks, int* redo, cudaStream_t s) {
+  static_assert(sizeof(FrameHeader) % 4 == 0, "copied by words");
+  const int grid = frame.nTiles > 0 ? (frame.nTiles + kOrderWarps - 1) / kOrderWarps : 1;
+  return launch_programmatic(k1_order_inline, grid, kOrderWarps * 32, 0, s, frame, hdr, srecs,
+                             blocks, redo);
 }
 
 // ----------------------------------------------------------------------------
