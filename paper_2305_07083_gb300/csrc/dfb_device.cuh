@@ -20,7 +20,6 @@ __device__ __forceinline__ uint32_t depth_bits(float z) {
   if (b == 0x80000000u) b = 0u;
   return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
-constexpr uint32_t kInfBits = 0xff800000u;  // depth_bits(+inf)
 
 __device__ __forceinline__ float2 e4m3x2_to_float2(uint32_t two_codes) {
   uint32_t h2;
