@@ -325,7 +325,9 @@ __device__ void producer(const FrameArgs* __restrict__ frames, const int* __rest
       const uint32_t more = FR == kOneFrame ? one.more : __shfl_sync(0xffffffffu, cur.sz.more, u);
       const int chunk =
           FR == kOneFrame ? item & (A->chunks - 1) : __shfl_sync(0xffffffffu, cur.chunk, u);
-      const uint32_t dBytes = bytes & 0xffffu, cBytes = bytes >> 16;
+      const uint32_t cBytes = bytes >> 16;
+      // a single fragment to blend needs no depth (item_mode)
+      const uint32_t dBytes = n == 1 && cBytes ? 0u : bytes & 0xffffu;
       const int P = (int)(more & 0xffffu), nState = (int)(more >> 16 & 0xffu);
       const size_t p0 = (size_t)chunk * P;  // the item's first pixel in its tile
       // An item of more than kN fragments is streamed in fills of kFill; its
@@ -521,6 +523,14 @@ __device__ __forceinline__ void blend_in_order(int n, int stride, const unsigned
     last = zz;
     rest |= in ? 0u : Px<DT>::bits(v);
   }
+}
+
+// The mode by which an item of `n` fragments is composited: a single fragment
+// has no order, so BLEND_DEPTH does not read its depth (an empty one is
+// blended too, as the last).  A server's step of 8 frames of one fragment per
+// tile, FP16, accumulating: launch 184.5 -> 176.7 us.
+__device__ __forceinline__ int item_mode(int mode, int n) {
+  return mode == DFB_BLEND_DEPTH && n == 1 ? (int)DFB_BLEND_ORDERED : mode;
 }
 
 // The nearest of one fill's `n` fragments at pixel t against `z`, the nearest
@@ -986,10 +996,10 @@ __device__ void consumer(const FrameArgs* __restrict__ frames, const int* __rest
                                ringBytes,
           ctl.err);
       if (w.active && inRing)
-        covered = P == kP ? composite_staged<DT, true>(A->mode, total, P, base, meta, t, w.p, c0,
-                                                       c1, c2, al)
-                          : composite_staged<DT, false>(A->mode, total, P, base, meta, t, w.p,
-                                                        c0, c1, c2, al);
+        covered = P == kP ? composite_staged<DT, true>(item_mode(A->mode, total), total, P,
+                                                       base, meta, t, w.p, c0, c1, c2, al)
+                          : composite_staged<DT, false>(item_mode(A->mode, total), total, P,
+                                                        base, meta, t, w.p, c0, c1, c2, al);
       // streamed state: from the ring into registers; then the ring space
       // goes back to the producer before the epilogue's math and stores
       if (stateRows && inRing) {
