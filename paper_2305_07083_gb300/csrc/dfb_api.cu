@@ -410,12 +410,16 @@ int allocate(dfb_ctx* h) {
   return st;
 }
 
-bool is_device_ptr(const void* p) {
+// Whether `p` is device (or managed) memory; `own`, if given: whether it is
+// ordinary memory of device `dev`, which that device's kernels can write.
+bool is_device_ptr(const void* p, int dev = -1, bool* own = nullptr) {
   cudaPointerAttributes at;
+  if (own) *own = false;
   if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
+  if (own) *own = at.type == cudaMemoryTypeDevice && at.device == dev;
   return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
@@ -1396,7 +1400,15 @@ namespace {
 // last frame; host destinations wait for completion.
 int copy_out(dfb_ctx* h, void* out, const void* src, size_t bytes) {
   cudaStream_t s = h->lastStream;
-  const bool dev = is_device_ptr(out);
+  bool own = false;
+  int current = -1;
+  const bool dev = is_device_ptr(out, h->device, &own);
+  if (own && (cudaGetDevice(&current) != cudaSuccess || current != h->device)) own = false;
+  // an image of this device's memory is copied by a kernel, which starts
+  // behind the frame's without the gap of a copy
+  if (own && (uintptr_t)out % 16 == 0 && bytes % 4 == 0)
+    return cuda_status(dfb::launch_copy(reinterpret_cast<const uint32_t*>(src),
+                                        reinterpret_cast<uint32_t*>(out), bytes / 4, s));
   cudaError_t e = cudaMemcpyAsync(out, src, bytes, dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess && !dev) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_status(e);

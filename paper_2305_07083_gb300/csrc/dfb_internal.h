@@ -218,6 +218,9 @@ constexpr double kStateLoadFragmentsPerTile = 2.0;
 //   out = (a - b) * scale  when b is given, else a * scale.
 cudaError_t launch_tiles_to_image(const float4* a, const float4* b, float scale, float4* out,
                                   int W, int H, int T, cudaStream_t s);
+// `words` 32-bit words from one device buffer to another, both 16-byte aligned
+// (at most 2^33 words).
+cudaError_t launch_copy(const uint32_t* src, uint32_t* dst, size_t words, cudaStream_t s);
 // Row-major image -> tile-major state (pixels outside the frame untouched).
 cudaError_t launch_image_to_tiles(const float4* in, float4* out, int W, int H, int T,
                                   cudaStream_t s);
