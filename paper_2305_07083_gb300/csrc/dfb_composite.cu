@@ -88,7 +88,7 @@ constexpr int kRound = 4;                // items the producer plans at once
 constexpr int kMetaQ = 2 * kRound;       // tile blocks fetched ahead
 constexpr uint32_t kWindowBytes = kSortWindow * kP * 8;
 constexpr int kRedoRank = 48;            // longest list the re-do kernel ranks
-constexpr int kRedoPer = 2;              // its CTAs per SM
+constexpr int kRedoPer = 3;              // its CTAs per SM
 
 // Descriptor of one fill of the ring: up to kN fragments of one work item
 // (all of them for an item of at most kN fragments, else kFill), and the
@@ -96,7 +96,7 @@ constexpr int kRedoPer = 2;              // its CTAs per SM
 struct __align__(16) ItemMeta {
   int n;               // fragments in this fill
   int total;           // fragments of the item
-  int first;           // list index of the fill's first fragment
+  int pad0;
   uint32_t start;      // byte offset of the fill's data in the ring
   uint32_t bytes;      // bytes of the fill's fragments from `start` (state rows follow)
   uint32_t end;        // producer's head count after this fill (modulo 2^32)
@@ -405,7 +405,7 @@ __device__ void producer(const FrameArgs* __restrict__ frames, const int* __rest
           if (DT == DFB_FP8E4M3) meta->scale[lane] = rScale;
         }
         if (lane == 0) {
-          *reinterpret_cast<int4*>(&meta->n) = make_int4(nf, n, i0, (int)start);
+          *reinterpret_cast<int4*>(&meta->n) = make_int4(nf, n, 0, (int)start);
           *reinterpret_cast<uint2*>(&meta->bytes) = make_uint2(fragBytes, head);
         }
         if (G > 1) {
@@ -649,9 +649,9 @@ __device__ __forceinline__ bool composite_staged(int mode, int n, int P, const u
 // list index) keys above the last one blended, blended in that order.  The
 // list arrives in (key, submit index) order, so ties on depth keep it.
 template <int DT>
-__device__ __forceinline__ void composite_exact(int n, const FragRec* list, uint64_t* kbAll,
-                                                int t, int p, float& c0, float& c1, float& c2,
-                                                float& al) {
+__device__ __noinline__ float4 composite_exact(int n, const FragRec* list, uint64_t* kbAll, int t,
+                                               int p) {
+  float c0 = 0.f, c1 = 0.f, c2 = 0.f, al = 0.f;
   uint64_t* kb = kbAll + t;
   uint64_t lo = 0;
   int done = 0;
@@ -699,6 +699,7 @@ __device__ __forceinline__ void composite_exact(int n, const FragRec* list, uint
     lo = last;
     done += m;
   }
+  return make_float4(c0, c1, c2, al);
 }
 
 // One pixel of one work item.
@@ -1115,13 +1116,13 @@ struct RedoWarp {
 template <int DT>
 __device__ __forceinline__ void composite_ranked(int n, RedoWarp* w, int lane, int p, float& c0,
                                                  float& c1, float& c2, float& al) {
-  for (int i0 = 0; i0 < n; i0 += 16) {
-    float z[16];
+  for (int i0 = 0; i0 < n; i0 += 8) {
+    float z[8];
 #pragma unroll
-    for (int u = 0; u < 16; ++u)
+    for (int u = 0; u < 8; ++u)
       if (i0 + u < n) z[u] = __ldg(w->depth[i0 + u] + p);
 #pragma unroll
-    for (int u = 0; u < 16; ++u)
+    for (int u = 0; u < 8; ++u)
       if (i0 + u < n) w->z[i0 + u][lane] = covers(z[u]) ? z[u] : INFINITY;
   }
   for (int i0 = 0; i0 < n; i0 += 4) {
@@ -1150,16 +1151,16 @@ __device__ __forceinline__ void composite_ranked(int n, RedoWarp* w, int lane, i
     for (int u = 0; u < 4; ++u)
       if (i0 + u < n) w->order[rank[u]][lane] = (unsigned char)(i0 + u);
   }
-  for (int r0 = 0; r0 < n; r0 += 8) {
-    float4 f[8];
+  for (int r0 = 0; r0 < n; r0 += 4) {
+    float4 f[4];
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
+    for (int u = 0; u < 4; ++u)
       if (r0 + u < n) {
         const int i = w->order[r0 + u][lane];
         f[u] = Px<DT>::global(w->rgba[i], p, w->scale[i]);
       }
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
+    for (int u = 0; u < 4; ++u)
       if (r0 + u < n) over(f[u], c0, c1, c2, al);
   }
 }
@@ -1174,11 +1175,15 @@ __device__ __forceinline__ void composite_ranked(int n, RedoWarp* w, int lane, i
 // the depths (bricks) there are no units and the kernel returns at once;
 // where producers overlap, most units of a long list are here.
 //
-// Bound by the latency of its dependent reads: 16 depths and 8 RGBA per lane
-// are in flight at a time.  1024x1024, FP32, 3,500 units of 17 to 24 fragments:
-// 31 us (41 us by windowed rounds; 41 us with 3 CTAs per SM, which spill).
-// Launched programmatically, so that a launch that finds no units costs no
-// more than its own start: 16 passes of FP8 4096x1024 1.435 -> 1.396 ms.
+// Bound by the latency of its dependent reads, so warps matter more than reads
+// in flight per warp: kRedoPer CTAs per SM (their scratch fills its shared
+// memory), 8 depths and 4 RGBA per lane at a time; the windowed rounds are a
+// call of their own, which keeps their registers out of the ranked path.  A
+// 1024x1024 FP32 frame with 3,500 units of 17 to 24 fragments takes 94.1 us
+// with its read-back; 100 us with 2 CTAs per SM and twice the reads in flight
+// or not; 41 against 31 us of this kernel by windowed rounds.  Launched
+// programmatically, so that a launch that finds no units costs no more than
+// its own start: 16 passes of FP8 4096x1024 1.435 -> 1.396 ms.
 template <int DT>
 __global__ void __launch_bounds__(kP, kRedoPer) k_composite_redo(
     const FrameArgs* __restrict__ frames, const int* __restrict__ itemBase, int nFrames,
@@ -1229,8 +1234,10 @@ __global__ void __launch_bounds__(kP, kRedoPer) k_composite_redo(
       __syncwarp();
     }
     if (__syncthreads_or(!ranked)) {
-      if (!ranked && w.active)
-        composite_exact<DT>(n, list, window, threadIdx.x, w.p, c0, c1, c2, al);
+      if (!ranked && w.active) {
+        const float4 v = composite_exact<DT>(n, list, window, threadIdx.x, w.p);
+        c0 = v.x; c1 = v.y; c2 = v.z; al = v.w;
+      }
       __syncthreads();
     }
     if (n > 0) {
