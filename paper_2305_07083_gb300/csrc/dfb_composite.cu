@@ -1250,23 +1250,9 @@ __global__ void __launch_bounds__(kP, kRedoPer) k_composite_redo(
   }
 }
 
-// Per-tile variance: one warp per global tile sums the tile's per-warp
+// Per-tile variance of one frame's tile: a warp sums the tile's per-warp
 // partials in slot order.
-__global__ void k_tile_variance(const FrameArgs* __restrict__ frames, int nFrames,
-                                int totalTiles) {
-  grid_dependency_wait();  // the composite's partials
-  allow_dependents();
-  const int gt = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5);
-  const int lane = threadIdx.x & 31;
-  if (gt >= totalTiles) return;
-  int lo = 0, hi = nFrames - 1;  // frame with the largest tileBase <= gt
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (frames[mid].tileBase <= gt) lo = mid; else hi = mid - 1;
-  }
-  const FrameArgs* A = frames + lo;
-  if (!(A->flags & DFB_FLAG_ACCUMULATE)) return;
-  const int tile = gt - A->tileBase;
+__device__ __forceinline__ void tile_variance(const FrameArgs* A, int tile, int lane) {
   const int slots = A->slots;
   float sum = 0.0f;
   for (int q = lane; q < slots; q += 32) sum += A->varPartial[(size_t)tile * slots + q];
@@ -1278,6 +1264,32 @@ __global__ void k_tile_variance(const FrameArgs* __restrict__ frames, int nFrame
     const int w = min(T, A->W - tx * T), h = min(T, A->H - ty * T);
     A->tileVar[tile] = sum / (3.0f * (float)(w * h));
   }
+}
+
+// One warp per global tile of a launch over several frames.
+__global__ void k_tile_variance(const FrameArgs* __restrict__ frames, int nFrames,
+                                int totalTiles) {
+  grid_dependency_wait();  // the composite's partials
+  allow_dependents();
+  const int gt = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5);
+  if (gt >= totalTiles) return;
+  int lo = 0, hi = nFrames - 1;  // frame with the largest tileBase <= gt
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (frames[mid].tileBase <= gt) lo = mid; else hi = mid - 1;
+  }
+  const FrameArgs* A = frames + lo;
+  if (A->flags & DFB_FLAG_ACCUMULATE) tile_variance(A, gt - A->tileBase, threadIdx.x & 31);
+}
+
+// The same for a single frame, whose arguments come with the launch: between
+// two composites this kernel is a chain of dependent loads, and the two from
+// the frame table are gone (16 passes of FP8 4096x1024 1.388 -> 1.382 ms).
+__global__ void k_tile_variance_one(const __grid_constant__ FrameArgs frame) {
+  grid_dependency_wait();
+  allow_dependents();
+  const int tile = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5);
+  if (tile < frame.nTiles) tile_variance(&frame, tile, threadIdx.x & 31);
 }
 
 template <int DT, int G, int PER>
@@ -1451,8 +1463,10 @@ cudaError_t launch_composite(const FrameArgs* frames, const int* itemBase, int n
     }
   }
   if (e != cudaSuccess || !accumulate || totalTiles < 1) return e;
-  return launch_programmatic(k_tile_variance, (totalTiles * 32 + 255) / 256, 256, 0, s, frames,
-                             nFrames, totalTiles);
+  const int grid = (totalTiles * 32 + 255) / 256;
+  if (hostFrames && nFrames == 1)
+    return launch_programmatic(k_tile_variance_one, grid, 256, 0, s, hostFrames[0]);
+  return launch_programmatic(k_tile_variance, grid, 256, 0, s, frames, nFrames, totalTiles);
 }
 
 }  // namespace dfb
