@@ -5,6 +5,7 @@
 // through an MPI messaging layer (Sec. 3, 3.2).  Here every tile is owned by
 // this process: setTile appends a 32-byte record to the frame's list, and at
 // end-of-frame the list is uploaded once and bucketed by tile on the GPU.
+#include <cuda.h>
 #include <math.h>
 #include <stdlib.h>
 #include <string.h>
@@ -421,6 +422,29 @@ bool is_device_ptr(const void* p, int dev = -1, bool* own = nullptr) {
   }
   if (own) *own = at.type == cudaMemoryTypeDevice && at.device == dev;
   return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
+}
+
+// Whether [p, p + bytes) lies inside the one allocation (or mapping) that `p`
+// points into.  False also where the driver cannot tell.
+bool in_one_allocation(const void* p, size_t bytes) {
+  using RangeOf = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+  static const RangeOf range_of = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault,
+                                         &found) != cudaSuccess ||
+        found != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return reinterpret_cast<RangeOf>(f);
+  }();
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  const CUdeviceptr at = (CUdeviceptr)(uintptr_t)p;
+  if (!range_of || range_of(&base, &size, at) != CUDA_SUCCESS || at < base) return false;
+  const size_t offset = (size_t)(at - base);
+  return offset <= size && bytes <= size - offset;
 }
 
 int validate_tile(const dfb_ctx* h, const dfb_tile_desc* t) {
@@ -1405,13 +1429,18 @@ int copy_out(dfb_ctx* h, void* out, const void* src, size_t bytes) {
   const bool dev = is_device_ptr(out, h->device, &own);
   if (own && (cudaGetDevice(&current) != cudaSuccess || current != h->device)) own = false;
   // an image of this device's memory is copied by a kernel, which starts
-  // behind the frame's without the gap of a copy
-  if (own && (uintptr_t)out % 16 == 0 && bytes % 4 == 0)
+  // behind the frame's without the gap of a copy.  The kernel checks nothing:
+  // a destination that is too small for the image is left to the copy, which
+  // the driver refuses.
+  if (own && (uintptr_t)out % 16 == 0 && bytes % 4 == 0 && in_one_allocation(out, bytes))
     return cuda_status(dfb::launch_copy(reinterpret_cast<const uint32_t*>(src),
                                         reinterpret_cast<uint32_t*>(out), bytes / 4, s));
   cudaError_t e = cudaMemcpyAsync(out, src, bytes, dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess && !dev) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) return cuda_status(e);
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // a refused copy is not the next launch's error
+    return cuda_status(e);
+  }
   return dev ? DFB_OK : take_device_error(h);
 }
 
