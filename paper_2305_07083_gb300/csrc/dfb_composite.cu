@@ -608,29 +608,36 @@ __device__ __forceinline__ bool composite_staged(int mode, int n, int P, const u
     // General case: sort of fragment indices (4-bit slots of `perm`) by
     // depth.  The list arrives in key order, so ties stay in (key, submit
     // index) order; empty fragments go to a second list kept in list order
-    // and blended last.  A finite fragment goes in front of the finite ones
-    // before it in the list that are deeper: they are counted, over all of
-    // the list so far, by loads that do not depend on one another (empty
-    // ones do not count).
+    // and blended last.  A finite fragment at least as deep as those before
+    // it goes to the end.  Another one goes in front of the finite ones before
+    // it that are deeper: all deeper depths in the list so far are counted, by
+    // loads that do not depend on one another, and the infinite ones (`far`)
+    // taken off.  In a list that is nearly in order few need the count:
+    // 2048x1024 FP16, 16 fragments of which two are swapped, 181 us, 244 with
+    // a count for each (random order, 1024x1024 FP32: 140 and 131).
     const float* zt = sD + t;
     uint64_t perm = 0, infs = 0;
-    int m = 0, mi = 0;
+    int m = 0, mi = 0, far = 0;
+    float deepest = -INFINITY;
     for (int i = 0; i < n; ++i) {
       const float z = zt[i * stride];
       const bool in = covers(z);
-      int deeper = 0;
+      int at = 4 * (in ? m : mi);
+      if (in && z < deepest) {
+        int deeper = -far;
 #pragma unroll 4
-      for (int j = 0; j < i; ++j) {
-        const float v = zt[j * stride];
-        deeper += covers(v) && v > z ? 1 : 0;
+        for (int j = 0; j < i; ++j) deeper += zt[j * stride] > z ? 1 : 0;
+        at -= 4 * deeper;
+        const uint64_t low = perm & ((1ull << at) - 1ull);
+        perm = low | ((perm ^ low) << 4);
       }
-      const int at = 4 * (m - deeper);
-      const uint64_t low = perm & ((1ull << at) - 1ull);
-      const uint64_t put = low | ((uint64_t)i << at) | ((perm ^ low) << 4);
-      perm = in ? put : perm;
-      infs |= in ? 0ull : (uint64_t)i << (4 * mi);
+      const uint64_t bit = (uint64_t)i << at;
+      perm |= in ? bit : 0ull;
+      infs |= in ? 0ull : bit;
+      deepest = in ? fmaxf(deepest, z) : deepest;
       m += in ? 1 : 0;
       mi += in ? 0 : 1;
+      far += z == INFINITY ? 1 : 0;
     }
     // one loop of exactly n steps: the finite list, then the empty ones
     for (int r = 0; r < n; ++r) {
