@@ -476,6 +476,12 @@ inline void count_frags(dfb_ctx* h, int tile, int c) {
   v += c;
 }
 
+// The open frame's long tiles, for the exact re-do that only BLEND_DEPTH needs.
+void add_long_tiles(const dfb_ctx* h, dfb::LongList& lng) {
+  if (h->cfg.mode != DFB_BLEND_DEPTH) return;
+  for (int t : h->longTiles) lng.add(h->fragCount[t], h->chunks);
+}
+
 void note_tree(dfb_ctx* h, int tile, int gen, int children) {
   if (gen == 1) {
     h->recvGen1[tile] += 1;
@@ -1206,11 +1212,8 @@ int end_one(dfb_ctx* h, cudaStream_t s) {
   hdr->itemBase[1] = h->nTiles * hdr->fa.chunks;
   const int items = hdr->itemBase[1];
   FrameHeader* dHdr = reinterpret_cast<FrameHeader*>(b.dStage);
-  // only BLEND_DEPTH items can need the exact re-do kernel
-  const int nLong = h->cfg.mode == DFB_BLEND_DEPTH ? (int)h->longTiles.size() : 0;
   dfb::LongList lng;
-  lng.items = nLong * h->chunks;
-  for (int t : h->longTiles) lng.maxFragments = std::max(lng.maxFragments, h->fragCount[t]);
+  add_long_tiles(h, lng);
   cudaError_t e = cudaSuccess;
   if (h->lastStreamSet && h->lastStream != s) e = cudaStreamWaitEvent(s, h->done, 0);
   cudaEvent_t* ev = timing_slot(h);
@@ -1251,7 +1254,7 @@ int end_one(dfb_ctx* h, cudaStream_t s) {
   if (e == cudaSuccess) e = cudaEventRecord(b.released, s);
   if (e == cudaSuccess) h->done = b.released;
   b.used = true;
-  h->launches += 1 + ((h->cfg.flags & DFB_FLAG_ACCUMULATE) ? 2 : 1) + (nLong ? 1 : 0);
+  h->launches += 1 + ((h->cfg.flags & DFB_FLAG_ACCUMULATE) ? 2 : 1) + lng.kernels();
   h->lastErr = h->errFlag;
   h->stallItem = -1;
   return cuda_status(e);
@@ -1308,8 +1311,7 @@ int end_batch(dfb_ctx* const* hs, int n, cudaStream_t s) {
       g.frame = (uint32_t)i;
       b.hRecs[b.cursor[g.tile]++] = g;
     }
-    if (h->cfg.mode == DFB_BLEND_DEPTH) lng.items += (int)h->longTiles.size() * h->chunks;
-    for (int t : h->longTiles) lng.maxFragments = std::max(lng.maxFragments, h->fragCount[t]);
+    add_long_tiles(h, lng);
     fill_frame_args(h, b.hFrames[i], tileBase, b.srecs, b.blocks);
     b.hItemBase[i] = items;
     items += h->nTiles * b.hFrames[i].chunks;
@@ -1347,7 +1349,7 @@ int end_batch(dfb_ctx* const* hs, int n, cudaStream_t s) {
                               ev ? ev[3] : nullptr, s);
   if (e == cudaSuccess) e = cudaEventRecord(b.released, s);
   b.used = true;
-  hs[0]->launches += 1 + (anyAcc ? 2 : 1) + (lng.items ? 1 : 0);
+  hs[0]->launches += 1 + (anyAcc ? 2 : 1) + lng.kernels();
   hs[0]->stallItem = -1;
   for (int i = 0; i < n && e == cudaSuccess; ++i) {
     e = cudaEventRecord(hs[i]->frameDone, s);
@@ -1748,8 +1750,7 @@ int graph_build(dfb_graph_t* g, const dfb_handle* hs, int n, dfb_graph* out) {
   for (int i = 0; i < n; ++i) {
     dfb_ctx* h = hs[i];
     g->anyAcc |= (h->cfg.flags & DFB_FLAG_ACCUMULATE) != 0;
-    if (h->cfg.mode == DFB_BLEND_DEPTH) g->lng.items += (int)h->longTiles.size() * h->chunks;
-    for (int t : h->longTiles) g->lng.maxFragments = std::max(g->lng.maxFragments, h->fragCount[t]);
+    add_long_tiles(h, g->lng);
     counts.insert(counts.end(), h->fragCount.begin(), h->fragCount.end());
     nRec += (int)h->recs.size();
     items += h->nTiles * h->chunks;
@@ -1888,7 +1889,7 @@ int dfb_graph_launch(dfb_graph g, void* stream) {
       h->lastStreamSet = true;
       h->haveFrame = true;
       h->lastErr = g->err;
-      h->launches += 1 + (g->anyAcc ? 2 : 1) + (g->lng.items ? 1 : 0);
+      h->launches += 1 + (g->anyAcc ? 2 : 1) + g->lng.kernels();
     }
     g->launched = true;
     return cuda_status(e);

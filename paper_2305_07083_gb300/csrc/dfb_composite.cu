@@ -87,8 +87,8 @@ constexpr int kSlots = 16;               // items in flight at most
 constexpr int kRound = 4;                // items the producer plans at once
 constexpr int kMetaQ = 2 * kRound;       // tile blocks fetched ahead
 constexpr uint32_t kWindowBytes = kSortWindow * kP * 8;
-constexpr int kRedoRank = 48;            // longest list the re-do kernel ranks
-constexpr int kRedoPer = 3;              // its CTAs per SM
+constexpr int kRedoPer = 3;              // CTAs per SM of the re-do, by ranks
+constexpr int kWindowPer = 3;            // and by windowed rounds
 
 // Descriptor of one fill of the ring: up to kN fragments of one work item
 // (all of them for an item of at most kN fragments, else kFill), and the
@@ -670,9 +670,9 @@ __device__ __forceinline__ bool composite_staged(int mode, int n, int P, const u
 // list index) keys above the last one blended, blended in that order.  The
 // list arrives in (key, submit index) order, so ties on depth keep it.
 template <int DT>
-__device__ __noinline__ float4 composite_exact(int n, const FragRec* list, uint64_t* kbAll, int t,
-                                               int p) {
-  float c0 = 0.f, c1 = 0.f, c2 = 0.f, al = 0.f;
+__device__ __forceinline__ void composite_exact(int n, const FragRec* list, uint64_t* kbAll,
+                                                int t, int p, float& c0, float& c1, float& c2,
+                                                float& al) {
   uint64_t* kb = kbAll + t;
   uint64_t lo = 0;
   int done = 0;
@@ -720,7 +720,6 @@ __device__ __noinline__ float4 composite_exact(int n, const FragRec* list, uint6
     lo = last;
     done += m;
   }
-  return make_float4(c0, c1, c2, al);
 }
 
 // One pixel of one work item.
@@ -1191,28 +1190,33 @@ __device__ __forceinline__ void composite_ranked(int n, RedoWarp* w, int lane, i
 // order at some pixel, or that had a non-zero empty fragment.  Each warp of a
 // CTA takes one unit at a time; each pixel reads its fragments from memory
 // (mostly still in L2) and blends them in exact (depth, key, submit index)
-// order -- by rank, or through the windowed rounds of composite_exact for the
-// longest lists -- then goes through the same epilogue.  Where the keys follow
-// the depths (bricks) there are no units and the kernel returns at once;
-// where producers overlap, most units of a long list are here.
+// order, then goes through the same epilogue.  Where the keys follow the
+// depths (bricks) there are no units and the kernel returns at once; where
+// producers overlap, most units of a long list are here.
 //
-// Bound by the latency of its dependent reads, so warps matter more than reads
-// in flight per warp: kRedoPer CTAs per SM (their scratch fills its shared
-// memory), 8 depths and 4 RGBA per lane at a time; the windowed rounds are a
-// call of their own, which keeps their registers out of the ranked path.  A
-// 1024x1024 FP32 frame with 3,500 units of 17 to 24 fragments takes 94.1 us
-// with its read-back; 100 us with 2 CTAs per SM and twice the reads in flight
-// or not; 41 against 31 us of this kernel by windowed rounds.  Launched
-// programmatically, so that a launch that finds no units costs no more than
-// its own start: 16 passes of FP8 4096x1024 1.435 -> 1.396 ms.
-template <int DT>
-__global__ void __launch_bounds__(kP, kRedoPer) k_composite_redo(
+// Two kernels, each for its own units; a launch runs those it has lists for:
+//   * RANKED: lists of up to kRedoRank fragments, by rank.  Bound by the
+//     latency of its dependent reads, so warps matter more than reads in
+//     flight per warp: kRedoPer CTAs per SM (their scratch fills its shared
+//     memory), 8 depths and 4 RGBA per lane at a time.  A 1024x1024 FP32 frame
+//     with 3,500 units of 17 to 24 fragments takes 88 us with its read-back;
+//     6 us more with 2 CTAs per SM and twice the reads in flight or not, or
+//     when the warps of a CTA wait for one another; 41 against 31 us of this
+//     kernel by windowed rounds.  Launched programmatically, so that a launch
+//     that finds no units costs no more than its own start: 16 passes of FP8
+//     4096x1024 1.435 -> 1.396 ms.
+//   * longer lists, by the windowed rounds of composite_exact.  As a call
+//     within the other kernel, whose warps then waited for one another, they
+//     were slower: a 512x512 FP32 frame out of order everywhere, 49 fragments
+//     per tile 704 us, 471 so; 150 per tile 4181 and 3173.  Launched plainly:
+//     with a programmatic launch, whose CTAs are placed while the composite
+//     still holds most SMs, the same frames take 640 and 3850 us.
+template <int DT, bool RANKED>
+__global__ void __launch_bounds__(kP, RANKED ? kRedoPer : kWindowPer) k_composite_redo(
     const FrameArgs* __restrict__ frames, const int* __restrict__ itemBase, int nFrames,
     LaunchCtl ctl) {
   extern __shared__ __align__(128) unsigned char lsmem[];
   SrgbTables* tb = reinterpret_cast<SrgbTables*>(lsmem);
-  RedoWarp* scratch = reinterpret_cast<RedoWarp*>(lsmem + sizeof(SrgbTables));
-  uint64_t* window = reinterpret_cast<uint64_t*>(scratch);  // longer lists, same memory
   grid_dependency_wait();  // the composite's list of units, and its writes
   allow_dependents();
   const int count = *(volatile int*)ctl.redo;
@@ -1220,31 +1224,22 @@ __global__ void __launch_bounds__(kP, kRedoPer) k_composite_redo(
   load_srgb(tb, kP);
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int u0 = blockIdx.x * kCW; u0 < count; u0 += gridDim.x * kCW) {
-    const int u = u0 + warp;
-    int n = 0, item = 0, iw = 0, f = 0, local = 0;
-    const FragRec* list = nullptr;
-    if (u < count) {
-      const int entry = ctl.redo[1 + u];
-      item = entry / kCW;
-      iw = entry % kCW;
-      f = find_frame(itemBase, nFrames, item);
-      local = item - __ldg(itemBase + f);
-      const FrameArgs* A = frames + f;
-      if (DFB_CHECK(f >= 0 && f < nFrames && (local >> A->logChunks) < A->nTiles, ctl.err)) {
-        const TileBlock* blk = A->blocks + A->tileBase + (local >> A->logChunks);
-        n = blk->n;
-        list = A->srecs + blk->off;
-      }
-    }
+  for (int u = blockIdx.x * kCW + warp; u < count; u += gridDim.x * kCW) {
+    const int entry = ctl.redo[1 + u];
+    const int item = entry / kCW, iw = entry % kCW;
+    const int f = find_frame(itemBase, nFrames, item);
+    const int local = item - __ldg(itemBase + f);
     const FrameArgs* A = frames + f;
+    if (!DFB_CHECK(f >= 0 && f < nFrames && (local >> A->logChunks) < A->nTiles, ctl.err))
+      continue;
+    const TileBlock* blk = A->blocks + A->tileBase + (local >> A->logChunks);
+    const int n = blk->n;
+    if ((n <= kRedoRank) != RANKED) continue;
+    const FragRec* list = A->srecs + blk->off;
     const PixWork w = prepare<kGlobalTable>(frames, itemBase, f, item, iw * 32 + lane);
     float c0 = 0.f, c1 = 0.f, c2 = 0.f, al = 0.f;
-    // A window column of one warp overlaps the scratch of others, so the CTA
-    // does its ranked units and its windowed ones one after the other.
-    const bool ranked = n <= kRedoRank;
-    if (n > 0 && ranked) {
-      RedoWarp* rw = scratch + warp;
+    if constexpr (RANKED) {
+      RedoWarp* rw = reinterpret_cast<RedoWarp*>(lsmem + sizeof(SrgbTables)) + warp;
       for (int i = lane; i < n; i += 32) {
         rw->rgba[i] = list[i].rgba;
         rw->depth[i] = list[i].depth;
@@ -1253,21 +1248,15 @@ __global__ void __launch_bounds__(kP, kRedoPer) k_composite_redo(
       __syncwarp();
       if (w.active) composite_ranked<DT>(n, rw, lane, w.p, c0, c1, c2, al);
       __syncwarp();
+    } else {
+      uint64_t* window = reinterpret_cast<uint64_t*>(lsmem + sizeof(SrgbTables));
+      if (w.active) composite_exact<DT>(n, list, window, threadIdx.x, w.p, c0, c1, c2, al);
     }
-    if (__syncthreads_or(!ranked)) {
-      if (!ranked && w.active) {
-        const float4 v = composite_exact<DT>(n, list, window, threadIdx.x, w.p);
-        c0 = v.x; c1 = v.y; c2 = v.z; al = v.w;
-      }
-      __syncthreads();
-    }
-    if (n > 0) {
-      const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
-      float4 S = zero4, M = zero4, CP = zero4;
-      if (w.active && (A->flags & DFB_FLAG_ACCUMULATE) && A->frameN != 1)
-        read_state<kGlobalTable>(A, w, S, M, CP);
-      finish_pixel<kGlobalTable>(A, w, lane, iw, c0, c1, c2, al, true, S, M, CP, tb, ctl.err);
-    }
+    const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 S = zero4, M = zero4, CP = zero4;
+    if (w.active && (A->flags & DFB_FLAG_ACCUMULATE) && A->frameN != 1)
+      read_state<kGlobalTable>(A, w, S, M, CP);
+    finish_pixel<kGlobalTable>(A, w, lane, iw, c0, c1, c2, al, true, S, M, CP, tb, ctl.err);
   }
 }
 
@@ -1371,8 +1360,38 @@ cudaError_t launch_shape(const FrameArgs* frames, const int* itemBase, int nFram
                              totalItems, ring, ctl, 0);
 }
 
-constexpr size_t kRedoBytes =
-    sizeof(RedoWarp) * kCW > kWindowBytes ? sizeof(RedoWarp) * kCW : kWindowBytes;
+constexpr int kRankedSmem = (int)(sizeof(SrgbTables) + sizeof(RedoWarp) * kCW);
+constexpr int kWindowSmem = (int)(sizeof(SrgbTables) + kWindowBytes);
+
+// One-time set-up of a format's re-do kernels on the current device.
+template <int DT>
+cudaError_t redo_setup() {
+  const cudaError_t e = cudaFuncSetAttribute(
+      k_composite_redo<DT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRankedSmem);
+  return e != cudaSuccess
+             ? e
+             : cudaFuncSetAttribute(k_composite_redo<DT, false>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, kWindowSmem);
+}
+
+// The re-do of a launch's long lists: at most one unit per warp of their
+// items; the count is on the device.
+template <int DT>
+cudaError_t launch_redo(const FrameArgs* frames, const int* itemBase, int nFrames,
+                        const LaunchCtl& ctl, const LongList& lng, int sms, cudaStream_t s) {
+  const int items = lng.ranked + lng.windowed;
+  auto grid = [&](int per) { return items < per * sms ? items : per * sms; };
+  cudaError_t e = cudaSuccess;
+  if (lng.ranked > 0)
+    e = launch_programmatic(k_composite_redo<DT, true>, grid(kRedoPer), kP, kRankedSmem, s, frames,
+                            itemBase, nFrames, ctl);
+  if (e == cudaSuccess && lng.windowed > 0) {
+    k_composite_redo<DT, false><<<grid(kWindowPer), kP, kWindowSmem, s>>>(frames, itemBase,
+                                                                         nFrames, ctl);
+    e = cudaGetLastError();
+  }
+  return e;
+}
 
 template <int DT>
 cudaError_t launch_dt(const FrameArgs* frames, const int* itemBase, int nFrames, int totalItems,
@@ -1442,46 +1461,21 @@ cudaError_t launch_composite(const FrameArgs* frames, const int* itemBase, int n
   int dev = 0;
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess && (dev < 0 || dev >= 64)) e = cudaErrorInvalidDevice;
-  const int smem = (int)(sizeof(SrgbTables) + kRedoBytes);
   if (e == cudaSuccess && !sms[dev]) {
     int count = 0;
     e = cudaDeviceGetAttribute(&count, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_composite_redo<DFB_F32>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_composite_redo<DFB_F16>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_composite_redo<DFB_BF16>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_composite_redo<DFB_FP8E4M3>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = redo_setup<DFB_F32>();
+    if (e == cudaSuccess) e = redo_setup<DFB_F16>();
+    if (e == cudaSuccess) e = redo_setup<DFB_BF16>();
+    if (e == cudaSuccess) e = redo_setup<DFB_FP8E4M3>();
     if (e == cudaSuccess) sms[dev] = count;
   }
-  if (e == cudaSuccess && lng.items > 0) {
-    // at most one unit per warp of the long items; the count is on the device
-    const int most = kRedoPer * sms[dev];
-    const int grid = lng.items < most ? lng.items : most;
-    switch (dtype) {
-      case DFB_F32:
-        e = launch_programmatic(k_composite_redo<DFB_F32>, grid, kP, smem, s, frames, itemBase,
-                                nFrames, ctl);
-        break;
-      case DFB_F16:
-        e = launch_programmatic(k_composite_redo<DFB_F16>, grid, kP, smem, s, frames, itemBase,
-                                nFrames, ctl);
-        break;
-      case DFB_BF16:
-        e = launch_programmatic(k_composite_redo<DFB_BF16>, grid, kP, smem, s, frames, itemBase,
-                                nFrames, ctl);
-        break;
-      default:
-        e = launch_programmatic(k_composite_redo<DFB_FP8E4M3>, grid, kP, smem, s, frames,
-                                itemBase, nFrames, ctl);
-        break;
-    }
+  if (e == cudaSuccess && lng.kernels()) {
+    auto redo = launch_redo<DFB_FP8E4M3>;
+    if (dtype == DFB_F32) redo = launch_redo<DFB_F32>;
+    if (dtype == DFB_F16) redo = launch_redo<DFB_F16>;
+    if (dtype == DFB_BF16) redo = launch_redo<DFB_BF16>;
+    e = redo(frames, itemBase, nFrames, ctl, lng, sms[dev], s);
   }
   if (e != cudaSuccess || !accumulate || totalTiles < 1) return e;
   const int grid = (totalTiles * 32 + 255) / 256;

@@ -130,12 +130,17 @@ struct TuneParams {
   int groups;     // consumer groups per CTA (items composited at once)
 };
 
-// Tiles of a launch with more than kStageFragments fragments: their work
-// items (the only ones that can need the exact re-do kernel) and the longest
-// list among them.
+// Longest list that the re-do kernel ranks; longer ones go in windowed rounds.
+constexpr int kRedoRank = 48;
+
+// Work items of a launch's BLEND_DEPTH tiles with more than kStageFragments
+// fragments, the only ones that can need an exact re-do, by the kernel that
+// would do it.
 struct LongList {
-  int items = 0;
-  int maxFragments = 0;
+  int ranked = 0;
+  int windowed = 0;
+  void add(int fragments, int items) { (fragments <= kRedoRank ? ranked : windowed) += items; }
+  int kernels() const { return (ranked > 0) + (windowed > 0); }
 };
 
 // An accumulating frame whose bytes exceed L2 would leave nothing of its state

@@ -144,12 +144,12 @@ int composite_noalloc(int width, int height, int tile_size, int mode, int dtype,
   FragRec* const recs = reinterpret_cast<FragRec*>(stage.get() + kHeaderBytes);
   int* const off = reinterpret_cast<int*>(recs + n);
   std::fill(off, off + nTiles + 1, 0);
-  int nLong = 0, maxFrags = 0;
+  int nLong = 0, nWindowed = 0;
   for (int i = 0; i < n; ++i) {
     if (tile_ids[i] < 0 || tile_ids[i] >= nTiles) return DFB_ERR_TILE_RANGE;
     const int c = ++off[tile_ids[i] + 1];
     if (c == dfb::kStageFragments + 1) ++nLong;
-    if (c > maxFrags) maxFrags = c;
+    if (c == dfb::kRedoRank + 1) ++nWindowed;
     if (isnan(order_keys[i]) || !rgba[i] || !depth[i]) return DFB_ERR_INVALID_ARG;
     if (((uintptr_t)rgba[i] % 16) || ((uintptr_t)depth[i] % 16)) return DFB_ERR_INVALID_ARG;
     if (dtype == DFB_FP8E4M3 && !(scales[i] > 0.0f && isfinite(scales[i])))
@@ -191,8 +191,10 @@ int composite_noalloc(int width, int height, int tile_size, int mode, int dtype,
   int* redo = reinterpret_cast<int*>(base + kOffRedo);
   Header* dHdr = reinterpret_cast<Header*>(base);
   dfb::LongList lng;
-  lng.items = (int)longItems;
-  lng.maxFragments = maxFrags;
+  if (longItems) {
+    lng.windowed = nWindowed * (int)chunksPerTile;
+    lng.ranked = (int)longItems - lng.windowed;
+  }
   // each record at its place in the list grouped by tile (stable: submission
   // order kept within a tile)
   const bool fp8 = dtype == DFB_FP8E4M3;

@@ -26,17 +26,23 @@ class Frame:
     def close(self):
         D.dfb_destroy(self.h)
 
-    def shortest(self, order, frames=40):
-        """Shortest composite of `frames` frames in ms, from the library's events around the launches."""
+    def shortest(self, order, frames=40, whole=False):
+        """Shortest composite of `frames` frames in ms, from the library's events around the launch; `whole`: all of a
+        frame's kernels, from events around its end."""
         import torch
         depth = order(self.j, self.r).expand(self.count, 4096).contiguous()
         rgba = D.pool_pointers(self.rgba, self.count, 4096 * 4 * D.ELEMENT_BYTES[self.dtype])
         z = D.pool_pointers(depth, self.count, 4096 * 4)
         torch.cuda.synchronize()
-        best = np.inf
+        best, s = np.inf, torch.cuda.Stream()
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         for _ in range(frames):
             D.dfb_begin_frame(self.h, 0)
             D.dfb_submit_tiles(self.h, self.ids, self.keys, rgba, z, None, D.DFB_PTR_DEVICE)
-            D.dfb_end_frame(self.h, None)
-            best = min(best, D.dfb_read_timing(self.h)["composite_ms"])
+            a.record(s)
+            D.dfb_end_frame(self.h, s)
+            b.record(s)
+            b.synchronize()
+            composite = D.dfb_read_timing(self.h)["composite_ms"]
+            best = min(best, a.elapsed_time(b) if whole else composite)
         return best
