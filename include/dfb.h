@@ -463,7 +463,8 @@ DFB_API int dfb_graph_destroy(dfb_graph g);
    shapes built are (groups, CTAs per SM) = (1, 2), (2, 2), (1, 3), (2, 1)
    and (3, 1).  0, 0, 0 restores the library default, chosen per launch:
    2 CTAs per SM with one group for FP32 and for single frames of 5 or more
-   fragment tiles per image tile, else 3 CTAs per SM.  A ring larger
+   fragment tiles per image tile (with a smaller ring up to 8), else 3 CTAs
+   per SM.  A ring larger
    than the CTAs can share is clamped at launch; one too small for the
    largest work item of the dtype makes the launch fail with DFB_ERR_CUDA.
    Errors: INVALID_ARG (a shape not in the list). */

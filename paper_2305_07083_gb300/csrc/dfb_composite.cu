@@ -1418,15 +1418,21 @@ cudaError_t launch_dt(const FrameArgs* frames, const int* itemBase, int nFrames,
 // the rings of 3.  The narrower formats' does, and 3 CTAs per SM are faster:
 // FP8 4096x1024, 3.4 fragments per tile, accumulating, 82 against 88 us; 16
 // mixed FP16 frames of 2 to 25 per tile in one launch 634 against 708 us.  The
-// exception is a single fragment-heavy frame, where the 2-CTA shape loads the
-// state one item ahead: FP16 2048x2048, 5.5 per tile, accumulating, 102.0
-// against 107.3 us (4.4 per tile: 102.8 against 94.5).  There a ring of 70 KB
-// beats the largest (103.6 us): more reads in flight than the DRAM queues
-// need only spread the accesses to a tile in time.  One CTA per SM is slower
-// everywhere: its single producer warp sets the pace.
+// exception are single FP16 and BF16 frames from 5 fragments per tile:
+// 2048x2048, 5.5 per tile, accumulating 102.0 against 107.3 us (4.4 per tile:
+// 102.8 against 94.5), not accumulating 6 per tile 90.9 against 97.7; FP8
+// would be faster with 3 there too (98 against 91 us).
+// A ring of 70 KB beats the largest (103.6 us) as long as it holds two items
+// and more: further reads in flight than the DRAM queues need only spread the
+// accesses to a tile in time.  At 8 per tile in every tile it takes 104 against
+// 112 us; at 12, where it holds one item, 167 against 132; in frames of bricks,
+// whose tiles differ, 117 and 117 at 7.7 per tile, 135 and 132 at 9.7, 154 and
+// 147 at 11.9.  So it is taken up to 8.  One CTA per SM is slower everywhere:
+// its single producer warp sets the pace.
 TuneParams default_tune(int dtype, double fragmentsPerTile, bool oneFrame) {
   if (dtype == DFB_F32) return TuneParams{110, 2, 1};
-  if (oneFrame && fragmentsPerTile >= 5.0) return TuneParams{70, 2, 1};
+  if (oneFrame && fragmentsPerTile >= 5.0)
+    return TuneParams{fragmentsPerTile <= 8.0 ? 70 : 110, 2, 1};
   return TuneParams{72, 3, 1};
 }
 
