@@ -11,6 +11,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <stdexcept>
@@ -97,6 +98,11 @@ unsigned long long g_table_devices = 0;  // bit d: table uploaded on device d
 
 }  // namespace
 
+// A device error word.  A launch over several handles, or of a graph, reports
+// through one word; every handle of it keeps the word until its next launch,
+// whatever is destroyed first.
+using ErrorWord = std::shared_ptr<unsigned>;
+
 // Device buffers of one frame's bucketing (K1) and its launch header.
 struct BucketSet {
   // [FrameHeader][FragRec x records, grouped by tile][tile offsets x nTiles+1],
@@ -154,8 +160,8 @@ struct dfb_ctx {
   int setIdx = 0;
   size_t recCap = 0;
   cudaStream_t bucketStream = nullptr;
-  unsigned* errFlag = nullptr;      // device error word of this handle's launches
-  unsigned* lastErr = nullptr;      // error word the last launch touching this handle used
+  ErrorWord errFlag;                // device error word of this handle's launches
+  ErrorWord lastErr;                // error word the last launch touching this handle used
   dfb::TuneParams tune{0, 0, 0};    // {0,0,0}: the library default
   unsigned long long waitNs = 2000000000ull;  // bound on every device-side wait
   int stallItem = -1;               // fault injection for tests (next launch only)
@@ -242,6 +248,19 @@ cudaError_t dalloc(T** p, size_t count) {
   return cudaMalloc(reinterpret_cast<void**>(p), sizeof(T) * (count ? count : 1));
 }
 
+// A new error word, clear.
+cudaError_t make_error_word(ErrorWord& w) {
+  unsigned* p = nullptr;
+  cudaError_t e = dalloc(&p, 1);
+  if (e != cudaSuccess) return e;
+  try {
+    w = ErrorWord(p, [](unsigned* q) { cudaFree(q); });  // frees p if it throws
+  } catch (const std::bad_alloc&) {
+    return cudaErrorMemoryAllocation;
+  }
+  return cudaMemset(p, 0, sizeof(unsigned));
+}
+
 // Upload buffer of one frame:
 //   [FrameHeader][FragRec x records, grouped by tile][tile offsets x nTiles+1]
 size_t stage_bytes(const dfb_ctx* h, size_t records) {
@@ -319,7 +338,9 @@ void free_device(dfb_ctx* h) {
   };
   fr(h->color); fr(h->accum); fr(h->comp); fr(h->m2); fr(h->rgba8);
   fr(h->tileVar); fr(h->varPartial);
-  fr(h->readTmp); fr(h->errFlag);
+  fr(h->readTmp);
+  h->errFlag.reset();
+  h->lastErr.reset();
   for (BucketSet& b : h->sets) {
     fr(b.redo);
     fr(b.dStage); fr(b.srecs); fr(b.blocks);
@@ -381,8 +402,7 @@ int allocate(dfb_ctx* h) {
   if (e == cudaSuccess && (f & DFB_FLAG_PACK_RGBA8)) e = dalloc(&h->rgba8, px);
   if (e == cudaSuccess) e = dalloc(&h->tileVar, h->nTiles);
   if (e == cudaSuccess) e = dalloc(&h->varPartial, (size_t)h->nTiles * ((h->tilePixels + 31) / 32));
-  if (e == cudaSuccess) e = dalloc(&h->errFlag, 1);
-  if (e == cudaSuccess) e = cudaMemset(h->errFlag, 0, sizeof(unsigned));
+  if (e == cudaSuccess) e = make_error_word(h->errFlag);
   if (e == cudaSuccess) e = cudaMemset(h->tileVar, 0, sizeof(float) * h->nTiles);
   for (BucketSet& b : h->sets) {
     if (e == cudaSuccess) e = dalloc(&b.blocks, h->nTiles);
@@ -672,7 +692,7 @@ dfb::TuneParams tune_of(const dfb_ctx* h, size_t nRec, size_t nTiles, bool oneFr
 }
 
 dfb::LaunchCtl ctl_of(const dfb_ctx* h, int* redo) {
-  return dfb::LaunchCtl{h->waitNs, h->stallItem, h->errFlag, redo};
+  return dfb::LaunchCtl{h->waitNs, h->stallItem, h->errFlag.get(), redo};
 }
 
 void finish_stats(dfb_ctx* h) {
@@ -1179,10 +1199,10 @@ cudaEvent_t* timing_slot(dfb_ctx* h) {
 int take_device_error(dfb_ctx* h) {
   if (!h->lastErr) return DFB_OK;
   unsigned v = 0;
-  cudaError_t e = cudaMemcpy(&v, h->lastErr, sizeof(unsigned), cudaMemcpyDeviceToHost);
+  cudaError_t e = cudaMemcpy(&v, h->lastErr.get(), sizeof(unsigned), cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_status(e);
   if (!v) return DFB_OK;
-  e = cudaMemset(h->lastErr, 0, sizeof(unsigned));
+  e = cudaMemset(h->lastErr.get(), 0, sizeof(unsigned));
   if (e != cudaSuccess) return cuda_status(e);
   return (v & dfb::kErrCheck) ? DFB_ERR_CHECK : DFB_ERR_TIMEOUT;
 }
@@ -1678,7 +1698,7 @@ struct dfb_graph_t {
   std::vector<int> hostItemBase;
   int* dItemBase = nullptr;
   dfb::LongList lng;
-  unsigned* err = nullptr;
+  ErrorWord err;
   dfb::TuneParams tune{0, 0, 0};
   cudaStream_t capStream = nullptr;
   cudaGraph_t graph = nullptr;
@@ -1706,7 +1726,7 @@ int graph_capture(dfb_graph_t* g) {
   graph_release_capture(g);
   const dfb::TuneParams tune = g->tune.ringKB ? g->tune : default_graph_tune(g);
   // per-device launch set-up happens outside the capture (no work is enqueued)
-  const dfb::LaunchCtl ctl{2000000000ull, -1, g->err, g->redo};
+  const dfb::LaunchCtl ctl{2000000000ull, -1, g->err.get(), g->redo};
   cudaError_t e = dfb::launch_composite(g->dFrames, g->dItemBase, 1, 0, 0, false, g->dtype, tune,
                                         ctl, dfb::LongList{}, nullptr, nullptr, nullptr,
                                         g->capStream);
@@ -1731,7 +1751,7 @@ void graph_free(dfb_graph_t* g) {
   graph_release_capture(g);
   cudaFree(g->dRecs); cudaFree(g->dOff); cudaFree(g->srecs); cudaFree(g->blocks);
   cudaFree(g->redo);
-  cudaFree(g->dFrames); cudaFree(g->dItemBase); cudaFree(g->err);
+  cudaFree(g->dFrames); cudaFree(g->dItemBase);
   if (g->capStream) cudaStreamDestroy(g->capStream);
   if (g->done) cudaEventDestroy(g->done);
   delete g;
@@ -1789,8 +1809,7 @@ int graph_build(dfb_graph_t* g, const dfb_handle* hs, int n, dfb_graph* out) {
   if (e == cudaSuccess) e = dalloc(&g->redo, (size_t)items * (dfb::kItemPixels / 32) + 1);
   if (e == cudaSuccess) e = dalloc(&g->dFrames, (size_t)n);
   if (e == cudaSuccess) e = dalloc(&g->dItemBase, (size_t)n + 1);
-  if (e == cudaSuccess) e = dalloc(&g->err, 1);
-  if (e == cudaSuccess) e = cudaMemset(g->err, 0, sizeof(unsigned));
+  if (e == cudaSuccess) e = make_error_word(g->err);
   if (e != cudaSuccess) {
     graph_free(g);
     return cuda_status(e);
