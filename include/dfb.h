@@ -158,7 +158,8 @@ typedef struct dfb_frame_stats {
   int64_t fragments;         /* tiles composited by the last frame            */
   int64_t fragment_pixels;   /* sum over fragments of in-frame pixels          */
   int64_t frame_pixels;      /* W * H                                          */
-  int64_t fragment_bytes;    /* algorithmic bytes of fragment data read        */
+  int64_t fragment_bytes;    /* algorithmic bytes of fragment data read (a
+                                tile's only fragment: without its depth)       */
   int64_t state_bytes;       /* algorithmic bytes of framebuffer state moved   */
   int32_t accumulated;       /* frames in the accumulation (1 after a reset)   */
   int32_t tiles;             /* tiles in the frame                             */

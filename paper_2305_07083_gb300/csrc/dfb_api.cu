@@ -695,6 +695,21 @@ dfb::LaunchCtl ctl_of(const dfb_ctx* h, int* redo) {
   return dfb::LaunchCtl{h->waitNs, h->stallItem, h->errFlag.get(), redo};
 }
 
+// In-frame pixels of the open frame's tiles with a single fragment.
+int64_t single_fragment_pixels(const dfb_ctx* h) {
+  const int T = h->cfg.tile_size;
+  int64_t px = 0;
+  const int* count = h->fragCount.data();
+  for (int ty = 0; ty < h->tilesY; ++ty, count += h->tilesX) {
+    const int64_t rows = std::min(T, h->cfg.height - ty * T);
+    int full = 0;
+    for (int tx = 0; tx + 1 < h->tilesX; ++tx) full += count[tx] == 1 ? 1 : 0;
+    const int last = h->cfg.width - (h->tilesX - 1) * T;  // width of the last column
+    px += rows * ((int64_t)full * T + (count[h->tilesX - 1] == 1 ? last : 0));
+  }
+  return px;
+}
+
 void finish_stats(dfb_ctx* h) {
   dfb_frame_stats& s = h->pendingStats;
   const int64_t px = (int64_t)h->cfg.width * h->cfg.height;
@@ -705,7 +720,8 @@ void finish_stats(dfb_ctx* h) {
   const int64_t rgbaPx = 4 * eb;
   if (h->cfg.mode == DFB_BLEND_ORDERED || h->cfg.mode == DFB_AVERAGE)
     s.fragment_bytes = s.fragment_pixels * rgbaPx;  // no depth read
-  else if (h->cfg.mode == DFB_BLEND_DEPTH) s.fragment_bytes = s.fragment_pixels * (rgbaPx + 4);
+  else if (h->cfg.mode == DFB_BLEND_DEPTH)  // a single fragment's depth is not read
+    s.fragment_bytes = s.fragment_pixels * (rgbaPx + 4) - single_fragment_pixels(h) * 4;
   else s.fragment_bytes = s.fragment_pixels * 4 + px * rgbaPx;  // depth + one winner
   int64_t st = 0;
   const unsigned f = h->cfg.flags;
