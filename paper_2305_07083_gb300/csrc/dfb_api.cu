@@ -194,6 +194,7 @@ namespace {
 
 int cuda_status(cudaError_t e) {
   if (e == cudaSuccess) return DFB_OK;
+  cudaGetLastError();  // returned here, so not the next launch's error too
   if (e == cudaErrorMemoryAllocation) return DFB_ERR_OOM;
   return DFB_ERR_CUDA;
 }
@@ -1475,11 +1476,15 @@ int copy_out(dfb_ctx* h, void* out, const void* src, size_t bytes) {
                                         reinterpret_cast<uint32_t*>(out), bytes / 4, s));
   cudaError_t e = cudaMemcpyAsync(out, src, bytes, dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess && !dev) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) {
-    cudaGetLastError();  // a refused copy is not the next launch's error
-    return cuda_status(e);
-  }
+  if (e != cudaSuccess) return cuda_status(e);
   return dev ? DFB_OK : take_device_error(h);
+}
+
+// Whether the kernels that read state back may write an image of `bytes` to
+// the caller's `out` themselves: device memory, aligned to their stores, that
+// the image fits into.  Any other destination gets a copy of the image.
+bool direct_image(const void* out, size_t bytes) {
+  return is_device_ptr(out) && (uintptr_t)out % 16 == 0 && in_one_allocation(out, bytes);
 }
 
 int ensure_read_tmp(dfb_ctx* h) {
@@ -1511,10 +1516,10 @@ int dfb_read_accum(dfb_handle h, float* out) {
   return guarded([&]() -> int {
     if (!h || !out) return DFB_ERR_INVALID_ARG;
     if (!h->haveFrame || !(h->cfg.flags & DFB_FLAG_ACCUMULATE)) return DFB_ERR_STATE;
-    const int64_t px = (int64_t)h->cfg.width * h->cfg.height;
-    const bool dev = is_device_ptr(out);
+    const size_t bytes = sizeof(float4) * (size_t)h->cfg.width * h->cfg.height;
+    const bool direct = direct_image(out, bytes);
     float4* dst = (float4*)out;
-    if (!dev) {
+    if (!direct) {
       const int st = ensure_read_tmp(h);
       if (st != DFB_OK) return st;
       dst = h->readTmp;
@@ -1524,8 +1529,7 @@ int dfb_read_accum(dfb_handle h, float* out) {
                                                1.0f / (float)n, dst, h->cfg.width, h->cfg.height,
                                                h->cfg.tile_size, h->lastStream);
     if (e != cudaSuccess) return cuda_status(e);
-    if (dev) return DFB_OK;
-    return copy_out(h, out, h->readTmp, sizeof(float4) * (size_t)px);
+    return direct ? DFB_OK : copy_out(h, out, h->readTmp, bytes);
   });
 }
 
@@ -1533,13 +1537,13 @@ int dfb_read_variance(dfb_handle h, float* per_pixel, float* per_tile) {
   return guarded([&]() -> int {
     if (!h) return DFB_ERR_INVALID_ARG;
     if (!h->haveFrame || !(h->cfg.flags & DFB_FLAG_ACCUMULATE)) return DFB_ERR_STATE;
-    const int64_t px = (int64_t)h->cfg.width * h->cfg.height;
+    const size_t bytes = sizeof(float4) * (size_t)h->cfg.width * h->cfg.height;
     const int n = h->accumN;
     const float invNm1 = n > 1 ? 1.0f / (float)(n - 1) : 0.0f;
     if (per_pixel) {
-      const bool dev = is_device_ptr(per_pixel);
+      const bool direct = direct_image(per_pixel, bytes);
       float4* dst = (float4*)per_pixel;
-      if (!dev) {
+      if (!direct) {
         const int st = ensure_read_tmp(h);
         if (st != DFB_OK) return st;
         dst = h->readTmp;
@@ -1547,8 +1551,8 @@ int dfb_read_variance(dfb_handle h, float* per_pixel, float* per_tile) {
       cudaError_t e = dfb::launch_tiles_to_image(h->m2, nullptr, invNm1, dst, h->cfg.width,
                                                  h->cfg.height, h->cfg.tile_size, h->lastStream);
       if (e != cudaSuccess) return cuda_status(e);
-      if (!dev) {
-        const int st = copy_out(h, per_pixel, h->readTmp, sizeof(float4) * (size_t)px);
+      if (!direct) {
+        const int st = copy_out(h, per_pixel, h->readTmp, bytes);
         if (st != DFB_OK) return st;
       }
     }
@@ -1576,9 +1580,10 @@ int dfb_get_tiles(dfb_handle h, int* tiles_x, int* tiles_y) {
 
 // Tile-major state buffer -> caller's row-major image (host or device).
 int state_out(dfb_ctx* h, float* out, const float4* src) {
-  const bool dev = is_device_ptr(out);
-  float4* dst = dev ? reinterpret_cast<float4*>(out) : nullptr;
-  if (!dev) {
+  const size_t bytes = sizeof(float4) * (size_t)h->cfg.width * h->cfg.height;
+  const bool direct = direct_image(out, bytes);
+  float4* dst = direct ? reinterpret_cast<float4*>(out) : nullptr;
+  if (!direct) {
     const int st = ensure_read_tmp(h);
     if (st != DFB_OK) return st;
     dst = h->readTmp;
@@ -1586,8 +1591,7 @@ int state_out(dfb_ctx* h, float* out, const float4* src) {
   cudaError_t e = dfb::launch_tiles_to_image(src, nullptr, 1.0f, dst, h->cfg.width, h->cfg.height,
                                              h->cfg.tile_size, h->lastStream);
   if (e != cudaSuccess) return cuda_status(e);
-  if (dev) return DFB_OK;
-  return copy_out(h, out, h->readTmp, sizeof(float4) * (size_t)h->cfg.width * h->cfg.height);
+  return direct ? DFB_OK : copy_out(h, out, h->readTmp, bytes);
 }
 
 int dfb_save_accum(dfb_handle h, float* sum, float* comp, float* m2, int* frames) {
