@@ -17,13 +17,15 @@
 // is to keep enough bytes in flight:
 //   * CTA = G consumer groups of 8 warps (one pixel per thread, 256 pixels =
 //     one work item; the groups take alternate items) + 1 producer warp, PER
-//     CTAs per SM (by default G = 1, PER = 2).  CTAs are persistent and walk
-//     the work items of all frames of the launch with a static stride, which
-//     keeps the chunks of a tile on neighbouring CTAs that run in step.
-//   * The producer warp fetches each item's tile block (fragment count,
-//     list offset and sorted records, written by the bucketing) with one bulk
-//     copy kMetaQ items ahead, so locating an item's fragments needs no
-//     dependent global loads.  It then issues one-dimensional bulk copies
+//     CTAs per SM (by default G = 1 and PER = 2 or 3, by default_tune).
+//     CTAs are persistent and walk the work items of all frames of the launch
+//     with a static stride, which keeps the chunks of a tile on neighbouring
+//     CTAs that run in step.
+//   * The producer warp takes its items in rounds of kRound.  It fetches a
+//     round's tile blocks (fragment count, list offset and sorted records,
+//     written by the bucketing) two rounds ahead, a bulk copy each and one
+//     barrier for all, so locating an item's fragments needs no dependent
+//     global loads.  It then issues one-dimensional bulk copies
 //     (cp.async.bulk, the TMA engine) of each fragment's depth slab and RGBA
 //     slab straight into a shared-memory ring, completing on the fill's
 //     mbarrier.  Fills take only the ring bytes they need (n fragments x slab
@@ -96,7 +98,7 @@ constexpr int kWindowPer = 3;            // and by windowed rounds
 struct __align__(16) ItemMeta {
   int n;               // fragments in this fill
   int total;           // fragments of the item
-  int pad0;
+  int pad0;            // n to start are one 16-byte store, bytes and end one of 8
   uint32_t start;      // byte offset of the fill's data in the ring
   uint32_t bytes;      // bytes of the fill's fragments from `start` (state rows follow)
   uint32_t end;        // producer's head count after this fill (modulo 2^32)
@@ -622,38 +624,51 @@ __device__ __forceinline__ bool composite_staged(int mode, int n, int P, const u
     // General case: sort of fragment indices (4-bit slots of `perm`) by
     // depth.  The list arrives in key order, so ties stay in (key, submit
     // index) order; empty fragments go to a second list kept in list order
-    // and blended last.  A finite fragment at least as deep as those before
-    // it goes to the end.  Another one goes in front of the finite ones before
-    // it that are deeper: all deeper depths in the list so far are counted, by
-    // loads that do not depend on one another, and the infinite ones (`far`)
-    // taken off.  In a list that is nearly in order few need the count:
-    // 2048x1024 FP16, 16 fragments of which two are swapped, 181 us, 244 with
-    // a count for each (random order, 1024x1024 FP32: 140 and 131).
+    // and blended last.  A finite fragment goes in front of the finite ones
+    // before it that are deeper: all deeper depths in the list so far are
+    // counted, by loads that do not depend on one another, and the infinite
+    // ones (`far`) taken off.  Two fragments share the loads, and a pair that
+    // is at least as deep as all before it needs no count, so that a list
+    // nearly in order costs little.  2048x1024 FP16, 16 fragments of which two
+    // are swapped, 174 us, 244 with a count for every fragment by itself;
+    // random order, 1024x1024 FP32, 123 and 131 (by insertion 176 and 252).
     const float* zt = sD + t;
     uint64_t perm = 0, infs = 0;
     int m = 0, mi = 0, far = 0;
     float deepest = -INFINITY;
-    for (int i = 0; i < n; ++i) {
-      const float z = zt[i * stride];
-      const bool in = covers(z);
-      int at = 4 * (in ? m : mi);
-      if (in && z < deepest) {
-        int deeper = -far;
-#pragma unroll 4
-        for (int j = 0; j < i; ++j) deeper += zt[j * stride] > z ? 1 : 0;
-        at -= 4 * deeper;
-        const uint64_t low = perm & ((1ull << at) - 1ull);
-        perm = low | ((perm ^ low) << 4);
-      }
-      const uint64_t bit = (uint64_t)i << at;
-      perm |= in ? bit : 0ull;
-      infs |= in ? 0ull : bit;
-      deepest = in ? fmaxf(deepest, z) : deepest;
+    auto place = [&](int i, bool in, int deeper) {
+      const int at = 4 * (m - (in ? deeper : 0));
+      const uint64_t low = perm & ((1ull << at) - 1ull);
+      const uint64_t put = low | ((uint64_t)i << at) | ((perm ^ low) << 4);
+      perm = in ? put : perm;
+      infs |= in ? 0ull : (uint64_t)i << (4 * mi);
       m += in ? 1 : 0;
       mi += in ? 0 : 1;
-      far += z == INFINITY ? 1 : 0;
+    };
+    for (int i = 0; i < n; i += 2) {
+      const bool two = i + 1 < n;
+      const float z0 = zt[i * stride];
+      const float z1 = two ? zt[(i + 1) * stride] : NAN;
+      const bool in0 = covers(z0), in1 = covers(z1);
+      const float mid = in0 ? fmaxf(deepest, z0) : deepest;
+      int d0 = 0, d1 = 0;
+      if ((in0 && z0 < deepest) || (in1 && z1 < mid)) {
+        d0 = -far;
+        d1 = in0 && z0 > z1 ? 1 - far : -far;
+#pragma unroll 2
+        for (int j = 0; j < i; ++j) {
+          const float v = zt[j * stride];
+          d0 += v > z0 ? 1 : 0;
+          d1 += v > z1 ? 1 : 0;
+        }
+      }
+      place(i, in0, d0);
+      if (two) place(i + 1, in1, d1);
+      deepest = in1 ? fmaxf(mid, z1) : mid;
+      far += (z0 == INFINITY ? 1 : 0) + (z1 == INFINITY ? 1 : 0);
     }
     // one loop of exactly n steps: the finite list, then the empty ones
+#pragma unroll 2
     for (int r = 0; r < n; ++r) {
       const bool fin = r < m;
       const uint64_t src = fin ? perm : infs;

@@ -1,6 +1,6 @@
 """GPU: staged BLEND_DEPTH lists that are nearly in order (a pair of fragments swapped), wholly out of it, and with
-empty fragments between: the sort counts only for a fragment nearer than one before it.  Lengths around the counting
-loop's remainders, up to the staged fill.
+empty fragments between: the sort takes two fragments at a time and counts only where one is nearer than one before it.
+Lengths around the pairs' and the counting loop's remainders, up to the staged fill.
 
 Tolerance: each of the n blends rounds a value of at most 1 three times, at most 1.5 n units of 2^-24 (n = 16: 1.5e-6).
 """
@@ -48,11 +48,11 @@ def test_swapped_pairs(n, order):
         fb.close()
 
 
-def test_nearly_sorted_lists_cost_less_than_random_ones():
-    """16 fragments of which the last two are swapped: 0.72 times the random frame's composite (as long as it, with a
-    count for every fragment)."""
+def test_cost_of_nearly_sorted_lists():
+    """16 fragments of which the last two are swapped take 1.5 times the composite of the frame in order (1.9 times,
+    with a count for every fragment by itself)."""
     f = Frame(16, D.DFB_F32)
     near = f.shortest(lambda j, r: j + 2.0 * (j == 14) - 1.0 * (j >= 14))
-    far = f.shortest(lambda j, r: r)
+    ordered = f.shortest(lambda j, r: j + 0.5 * r)
     f.close()
-    assert near <= 0.87 * far
+    assert near <= 1.7 * ordered
